@@ -6,13 +6,15 @@
 //   3. training sets: one CTA per cell gathers the samples of the neighbouring cells that fall in its
 //      collection box [o + c h - mu, o + (c+1) h + mu) (binary64 compares), sorts them by global id in
 //      shared memory and keeps ranks floor(j cnt / n_max) when there are more than n_max;
-//   4. the fit: A = K + diag(sigma^2) with K_ij = exp(-lambda |x_i - x_j|^2) in FP64, the FP64 Cholesky
-//      factor A = L L^T (blocked, right looking) and alpha = A^{-1} 1 by two FP64 triangular solves (all
-//      labels are 1); L^{-1} for the variance contraction in FP32, from L rounded to FP32.  Persistent
-//      CTAs take the cells in descending size order, in four size classes launched concurrently: the
-//      packed matrix lives in shared memory up to N = 218 and in a per-CTA global scratch slot above that.
+//   4. the fit: A = K + diag(sigma^2) with K_ij = exp(-lambda |x_i - x_j|^2) to binary64 accuracy, the
+//      Cholesky factor A = L L^T and alpha = A^{-1} 1 by two triangular solves (all labels are 1);
+//      L^{-1} for the variance contraction in FP32, from L rounded to FP32.  Cells whose variances allow it
+//      are factored in 64-bit fixed point (ksdf_fixchol.cuh), the others in binary64 (k_fit: blocked, right
+//      looking).  Persistent CTAs take the cells in descending size order, in size classes launched
+//      concurrently; the packed matrix lives in shared memory, or in a per-CTA global slot for the largest.
 #include "ksdf_exp.cuh"
 #include "ksdf_internal.cuh"
+#include "ksdf_fixchol.cuh"
 
 #include <cmath>
 #include <cstdarg>
@@ -301,12 +303,28 @@ __global__ void k_sched_after(const int32_t* touched, int64_t G, int32_t* c0, in
   }
 }
 
-__global__ void k_order_keys(const int32_t* n32, const int32_t* touched, int64_t G, int n_max, uint64_t* keys,
-                             uint32_t* vals) {
-  int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// The fit order's sort key of each cell (a warp per cell): cells for the fixed-point factorisation (fx allowed and
+// every sigma_i^2 within its bounds) by descending size, then the cells for the binary64 one by descending size,
+// then the cells that are not fitted; hist[0 .. n_max] counts the first kind by size, hist[n_max + 1 ..] the second.
+__global__ void k_order_keys(const int32_t* n32, const int32_t* touched, const int64_t* ts_off, const float* mvar,
+                             int64_t G, int n_max, int fx, uint64_t* keys, uint32_t* vals, int* hist) {
+  const int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
   if (g >= G) return;
-  keys[g] = (!touched || touched[g]) ? (uint64_t)(n_max - n32[g]) : (uint64_t)(n_max + 1);
-  vals[g] = (uint32_t)g;
+  const int n = n32[g];
+  const bool fit = !touched || touched[g];
+  bool ok = fx != 0 && n > 0;
+  if (fit && ok) {
+    const float* v = mvar + ts_off[g];
+    for (int i = lane; i < n; i += 32) ok &= v[i] >= kFxMinVar && v[i] <= kFxMaxVar;
+  }
+  ok = __all_sync(0xffffffffu, ok);
+  if (lane == 0) {
+    const int base = ok ? 0 : n_max + 1;
+    keys[g] = fit ? (uint64_t)(base + n_max - n) : (uint64_t)(2 * (n_max + 1));
+    vals[g] = (uint32_t)g;
+    if (fit) atomicAdd(&hist[base + n], 1);
+  }
 }
 
 // update: touched[g] = 1 unless the previous model has a cell with the same key, an OK fit and the same
@@ -435,15 +453,8 @@ struct KmatArgs {
   double sc;   // sqrt(lambda 2^16 / ln2): coordinates scaled so that |s_i - s_j|^2 is exp2_neg_q16's argument
   float lamf;  // lambda in FP32 (the near/far screen)
   bool fixed;  // scaled coordinates below 2^21: exact fixed-point squared distances (else binary64)
+  int64_t nfx; // the first nfx cells get their entries in Q60 (the fixed-point factorisation's input)
 };
-
-// row of the packed lower-triangle entry t (t = i (i+1)/2 + j, j <= i)
-__device__ __forceinline__ int tri_row(int64_t t) {
-  int i = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
-  while (tri_sz(i + 1) <= t) ++i;
-  while (tri_sz(i) > t) --i;
-  return i;
-}
 
 constexpr int kB = 8;        // Cholesky panel width
 constexpr float kNearE = 36.f;  // RBF: lambda r^2 below this: FP64 entry; above: FP32 (value < 2.4e-16)
@@ -513,6 +524,10 @@ __global__ void __launch_bounds__(32 * kKmatWarps) k_kmat(KmatArgs a) {
     const int N = a.n32[g];
     const int64_t m0 = a.ts_off[g];
     double* Ag = a.chol64 + a.chol_off[g];
+    const bool q60 = w < a.nfx;
+    auto put = [&](int i, int j, double v) {
+      Ag[tri_sz(i) + j] = q60 ? __longlong_as_double(fx_from_double(v)) : v;
+    };
     for (int i = lane; i < N; i += 32) {
       const D4 v = a.md4[m0 + i];
       const double sv[3] = {a.sc * v.x, a.sc * v.y, a.sc * v.z};
@@ -524,7 +539,7 @@ __global__ void __launch_bounds__(32 * kKmatWarps) k_kmat(KmatArgs a) {
       xf[4 * i] = f.x;
       xf[4 * i + 1] = f.y;
       xf[4 * i + 2] = f.z;
-      Ag[tri_sz(i) + i] = 1.0 + f2d_bits(a.mvar[m0 + i]);  // exp(0) + sigma_i^2
+      put(i, i, 1.0 + f2d_bits(a.mvar[m0 + i]));  // exp(0) + sigma_i^2
     }
     __syncwarp();
     // the strictly lower pairs flattened, t = i (i - 1) / 2 + j, 32 consecutive pairs per step (full warps
@@ -545,11 +560,11 @@ __global__ void __launch_bounds__(32 * kKmatWarps) k_kmat(KmatArgs a) {
         if (MATERN) {
           const float ef = a.lamf * sqrtf(fmaf(dz, dz, fmaf(dy, dy, dx * dx)));
           if (ef < kNearM) near = true;
-          else Ag[tri_sz(i) + j] = f2d_bits((1.f + ef) * exp2f(-1.44269504f * ef));
+          else put(i, j, f2d_bits((1.f + ef) * exp2f(-1.44269504f * ef)));
         } else {
           const float ef = a.lamf * fmaf(dz, dz, fmaf(dy, dy, dx * dx));
           if (ef < kNearE) near = true;
-          else Ag[tri_sz(i) + j] = f2d_bits(exp2f(-1.44269504f * ef));
+          else put(i, j, f2d_bits(exp2f(-1.44269504f * ef)));
         }
       }
       const unsigned mask = __ballot_sync(0xffffffffu, near);
@@ -558,7 +573,7 @@ __global__ void __launch_bounds__(32 * kKmatWarps) k_kmat(KmatArgs a) {
       if (qn >= 32) {
         __syncwarp();
         const int ij = qw[lane];
-        Ag[tri_sz(ij >> 16) + (ij & 0xffff)] = near_entry<MATERN>(s, sfix, a.fixed, ij >> 16, ij & 0xffff);
+        put(ij >> 16, ij & 0xffff, near_entry<MATERN>(s, sfix, a.fixed, ij >> 16, ij & 0xffff));
         __syncwarp();
         if (lane < qn - 32) qw[lane] = qw[32 + lane];
         qn -= 32;
@@ -573,7 +588,7 @@ __global__ void __launch_bounds__(32 * kKmatWarps) k_kmat(KmatArgs a) {
     __syncwarp();
     if (lane < qn) {
       const int ij = qw[lane];
-      Ag[tri_sz(ij >> 16) + (ij & 0xffff)] = near_entry<MATERN>(s, sfix, a.fixed, ij >> 16, ij & 0xffff);
+      put(ij >> 16, ij & 0xffff, near_entry<MATERN>(s, sfix, a.fixed, ij >> 16, ij & 0xffff));
     }
     __syncwarp();
   }
@@ -1255,7 +1270,7 @@ static int bits_for(uint64_t v) {
 
 // persistent launches of one size class: as many teams as fit on the GPU (at most one per cell)
 template <class K, class Args, class... Extra>
-static cudaError_t launch_persistent(ksdf_ctx* c, K kern, int team, const Args& f, size_t smem, bool gslot,
+static cudaError_t launch_persistent(ksdf_ctx* c, K kern, int team, const Args& f, size_t smem, int gslots,
                                      cudaStream_t s, const Extra&... extra) {
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -1263,7 +1278,7 @@ static cudaError_t launch_persistent(ksdf_ctx* c, K kern, int team, const Args& 
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, team, smem);
   if (e != cudaSuccess) return e;
   int64_t nblk = std::min<int64_t>(f.count, (int64_t)std::max(1, occ) * c->num_sms);
-  if (gslot) nblk = std::min<int64_t>(nblk, c->num_sms);  // one global slot per CTA
+  if (gslots) nblk = std::min<int64_t>(nblk, (int64_t)gslots * c->num_sms);  // one global slot per CTA
   launch(kern, (unsigned)nblk, team, smem, s, f, extra...);
   return cudaSuccess;
 }
@@ -1466,37 +1481,37 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
            ptr<int64_t>(m.ts_off), ptr<int32_t>(m.mgid), G, ptr<uint64_t>(o.hkeys), ptr<int32_t>(o.hvals), o.hcap,
            ptr<int32_t>(o.n), ptr<int64_t>(o.ts_off), ptr<int32_t>(o.mgid), ptr<int32_t>(o.status), touched, oid);
   }
-  launch(k_order_keys, ceil_div(G, 256), 256, 0, st, ptr<int32_t>(m.n), touched, G, p.n_max, okeys, order);
-  KSDF_CUDA(c, radix_sort_u64(okeys, order, G, bits_for((uint64_t)p.n_max + 1), c->ws[WS_SORT], st));
-  // size classes (host histogram of the cells to fit), launched concurrently, largest first; each class has
-  // its team size
-  std::vector<int32_t> hn((size_t)G), ht;
-  KSDF_CUDA(c, cudaMemcpyAsync(hn.data(), m.n.p, sizeof(int32_t) * G, cudaMemcpyDeviceToHost, st));
-  if (prev) {
-    ht.resize((size_t)G);
-    KSDF_CUDA(c, cudaMemcpyAsync(ht.data(), touched, sizeof(int32_t) * G, cudaMemcpyDeviceToHost, st));
-  }
+  const int nh = 2 * (p.n_max + 1);
+  KSDF_CUDA(c, ensure(c->ws[WS_E], sizeof(int64_t) * 4 + sizeof(int) * (64 + 2 * (kMaxNmax + 1))));
+  int* ctr = reinterpret_cast<int*>(ptr<int64_t>(c->ws[WS_E]) + 4);  // counters of the persistent launches
+  int* dhist = ctr + 64;
+  KSDF_CUDA(c, cudaMemsetAsync(ctr, 0, sizeof(int) * (64 + nh), st));
+  launch(k_order_keys, ceil_div(G * 32, 256), 256, 0, st, ptr<int32_t>(m.n), touched, ptr<int64_t>(m.ts_off),
+         ptr<float>(m.mvar), G, p.n_max, 1, okeys, order, dhist);
+  KSDF_CUDA(c, radix_sort_u64(okeys, order, G, bits_for((uint64_t)nh), c->ws[WS_SORT], st));
+  // size classes from the counts by kind and size, launched concurrently, largest first; each class has its team size
+  std::vector<int> hist((size_t)nh);
+  KSDF_CUDA(c, cudaMemcpyAsync(hist.data(), dhist, sizeof(int) * nh, cudaMemcpyDeviceToHost, st));
   KSDF_CUDA(c, cudaStreamSynchronize(st));
   int64_t nfit = 0;
-  for (int64_t g = 0; g < G; ++g) {
-    if (prev && !ht[(size_t)g]) hn[(size_t)g] = -1;  // not fitted: out of every class
-    else ++nfit;
-  }
+  for (int v : hist) nfit += v;
   if (n_refit) *n_refit = nfit;
-  using FitClass = FitClassCfg;
-  const std::vector<FitClassCfg>& cls = c->fit_cls.empty() ? fit_table(0) : c->fit_cls;
-  const int kNumClass = (int)cls.size();
-  std::vector<int64_t> cnt((size_t)kNumClass, 0);
-  for (int32_t v : hn) {
-    if (v < 0) continue;
-    int cl = kNumClass - 1;
-    while (cl > 0 && v > cls[cl].np) --cl;
-    ++cnt[cl];
+  struct Class {
+    FitClassCfg cfg;
+    bool fx;
+    int64_t count;
+  };
+  std::vector<Class> classes;
+  for (int kind = 0; kind < 2; ++kind) {
+    const std::vector<FitClassCfg>& t = kind == 0 ? fit_table(c->fit_tab).fx : fit_table(c->fit_tab).f64;
+    for (size_t i = 0; i < t.size(); ++i) {
+      const int lo = i + 1 < t.size() ? t[i + 1].np + 1 : 0, hi = std::min(t[i].np, p.n_max);
+      Class cl{t[i], kind == 0, 0};
+      for (int n = lo; n <= hi; ++n) cl.count += hist[(size_t)(kind * (p.n_max + 1) + n)];
+      classes.push_back(cl);
+    }
   }
   KSDF_CUDA(c, cudaMemsetAsync(dmax, 0, sizeof(int) * 2, st));
-  KSDF_CUDA(c, ensure(c->ws[WS_E], sizeof(int64_t) * 4 + sizeof(int) * 32));  // counters: fit and L^-1 classes
-  int* ctr = reinterpret_cast<int*>(ptr<int64_t>(c->ws[WS_E]) + 4);
-  KSDF_CUDA(c, cudaMemsetAsync(ctr, 0, sizeof(int) * 32, st));
   FitArgs fa;
   fa.order = order;
   fa.n32 = ptr<int32_t>(m.n);
@@ -1514,12 +1529,15 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
   fa.gstride = 0;
   // kernel matrices of the cells to fit (largest first), into the factor's place
   e0 = prof_begin(c);
+  int64_t nfx = 0;
+  for (int n = 0; n <= p.n_max; ++n) nfx += hist[(size_t)n];
   if (nfit > 0) {
     KmatArgs ka;
+    ka.nfx = nfx;
     ka.order = order;
     ka.first = 0;
     ka.count = nfit;
-    ka.counter = ctr + 24;
+    ka.counter = ctr + 32;
     ka.n32 = ptr<int32_t>(m.n);
     ka.ts_off = ptr<int64_t>(m.ts_off);
     ka.chol_off = ptr<int64_t>(m.chol_off);
@@ -1546,36 +1564,85 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
   KSDF_CUDA(c, fork_streams(c));
   int64_t first = 0;
   int launched = 0;
-  for (int cl = 0; cl < kNumClass; ++cl) {
-    if (cnt[cl] == 0) continue;
-    FitArgs f = fa;
-    f.first = first;
-    f.count = cnt[cl];
-    f.counter = ctr + cl;
-    first += cnt[cl];
-    const int team = cls[cl].team;
-    f.np = cls[cl].gmat ? std::max(m.max_n, 1) : cls[cl].np;
-    const size_t smem = sizeof(double) * (size_t)(fit_smem_doubles(f.np, !cls[cl].gmat) +
-                                                  (cls[cl].gmat ? (int64_t)(f.np + 1) * kB : 0));
+  for (size_t cl = 0; cl < classes.size(); ++cl) {
+    const FitClassCfg& cfg = classes[cl].cfg;
+    if (classes[cl].count == 0) continue;
+    const int team = cfg.team;
+    const int np = cfg.gmat ? std::min(std::max(m.max_n, 1), cfg.np) : cfg.np;
     const int si = launched % ksdf_ctx::kNumAux;  // auxiliary streams only: the main stream marks the stage end
     cudaStream_t s = c->aux[si];
     ++launched;
-    if (cls[cl].gmat) {
-      f.gstride = tri_sz(f.np + 1);
-      const int64_t slots = std::min<int64_t>(cnt[cl], c->num_sms);
-      KSDF_CUDA(c, ensure(c->ws[WS_FITSCR], sizeof(double) * (size_t)(f.gstride * slots + 1)));
-      f.gscr = ptr<double>(c->ws[WS_FITSCR]);
-    }
     cudaError_t le = cudaSuccess;
-    switch (team) {
-      case 256: le = cls[cl].gmat ? launch_persistent(c, k_fit<256, true>, 256, f, smem, true, s, p)
-                                  : launch_persistent(c, k_fit<256, false>, 256, f, smem, false, s, p); break;
-      case 128: le = launch_persistent(c, k_fit<128, false>, 128, f, smem, false, s, p); break;
-      case 64: le = launch_persistent(c, k_fit<64, false>, 64, f, smem, false, s, p); break;
-      default: le = launch_persistent(c, k_fit<32, false>, 32, f, smem, false, s, p); break;
+    FitArgs f = fa;
+    f.first = first;
+    f.count = classes[cl].count;
+    f.counter = ctr + cl;
+    f.np = np;
+    first += f.count;
+    if (classes[cl].fx) {
+      FixArgs x;
+      x.order = order;
+      x.first = f.first;
+      x.count = f.count;
+      x.counter = f.counter;
+      x.n32 = f.n32;
+      x.ts_off = f.ts_off;
+      x.chol_off = f.chol_off;
+      x.md4 = f.md4;
+      x.chol64 = f.chol64;
+      x.gscr = nullptr;
+      x.gstride = 0;
+      x.np = np;
+      x.st = stw;
+      const size_t smem = team == 32 ? 8 * (size_t)fx_elems(np + 1) : fx_team_smem(np, !cfg.gmat, team / 32);
+      if (cfg.gmat) {
+        x.gstride = fx_elems(np + 1);
+        const int64_t slots = std::min<int64_t>(f.count, (team == 512 ? 1 : 2) * c->num_sms);
+        DevBuf& scr = c->ws[team == 512 ? WS_FIXSCR : WS_FIXSCR2];
+        KSDF_CUDA(c, ensure(scr, sizeof(int2) * (size_t)(x.gstride * slots + 2)));
+        x.gscr = ptr<int2>(scr);
+      }
+      switch (team) {
+        case 512: le = launch_persistent(c, k_fit_fx<16, true>, team, x, smem, 1, s); break;
+        case 256: le = launch_persistent(c, k_fit_fx<8, true>, team, x, smem, 2, s); break;
+        case 224: le = launch_persistent(c, k_fit_fx<7, false>, team, x, smem, 0, s); break;
+        case 160: le = launch_persistent(c, k_fit_fx<5, false>, team, x, smem, 0, s); break;
+        case 128: le = launch_persistent(c, k_fit_fx<4, false>, team, x, smem, 0, s); break;
+        default: le = launch_persistent(c, k_fit_fx1, 32, x, smem, 0, s); break;
+      }
+    } else {
+      const size_t smem =
+          sizeof(double) * (size_t)(fit_smem_doubles(np, !cfg.gmat) + (cfg.gmat ? (int64_t)(np + 1) * kB : 0));
+      if (cfg.gmat) {
+        f.gstride = tri_sz(np + 1);
+        const int64_t slots = std::min<int64_t>(f.count, c->num_sms);
+        KSDF_CUDA(c, ensure(c->ws[WS_FITSCR], sizeof(double) * (size_t)(f.gstride * slots + 1)));
+        f.gscr = ptr<double>(c->ws[WS_FITSCR]);
+      }
+      switch (team) {
+        case 256: le = cfg.gmat ? launch_persistent(c, k_fit<256, true>, 256, f, smem, 1, s, p)
+                                : launch_persistent(c, k_fit<256, false>, 256, f, smem, 0, s, p); break;
+        case 128: le = launch_persistent(c, k_fit<128, false>, 128, f, smem, 0, s, p); break;
+        case 64: le = launch_persistent(c, k_fit<64, false>, 64, f, smem, 0, s, p); break;
+        default: le = launch_persistent(c, k_fit<32, false>, 32, f, smem, 0, s, p); break;
+      }
     }
     KSDF_CUDA(c, le);
     KSDF_CUDA(c, cudaEventRecord(c->ev_mid[si], s));
+    if (classes[cl].fx) {
+      AlphaArgs aa;
+      aa.order = order;
+      aa.first = f.first;
+      aa.count = f.count;
+      aa.n32 = f.n32;
+      aa.ts_off = f.ts_off;
+      aa.chol_off = f.chol_off;
+      aa.md4 = f.md4;
+      aa.mf4 = f.mf4;
+      aa.chol64 = f.chol64;
+      auto ka = np <= 64 ? k_alpha<2> : np <= 96 ? k_alpha<3> : np <= 128 ? k_alpha<4> : np <= 256 ? k_alpha<8> : k_alpha<16>;
+      launch(ka, ceil_div(f.count, kAlphaWarps), 32 * kAlphaWarps, 0, s, aa);
+    }
     // L^{-1} in FP32 of the same cells, behind their factorisation, on a high-priority stream: its blocks take
     // the SM resources this class's factorisation frees ahead of the pending blocks of the other classes'
     // factorisations, so that its FP32 work overlaps their FP64 work instead of trailing it
@@ -1599,17 +1666,17 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
       la.gstride = 0;
       la.np = f.np;
       if (f.np <= 96) {
-        le = launch_persistent(c, k_linv_small<1>, 32, la, sizeof(float) * (size_t)linv_small_floats(f.np, 1), false,
+        le = launch_persistent(c, k_linv_small<1>, 32, la, sizeof(float) * (size_t)linv_small_floats(f.np, 1), 0,
                                sh);
       } else if (f.np <= kTcMaxN) {
-        le = launch_persistent(c, k_linv_small<2>, 64, la, sizeof(float) * (size_t)linv_small_floats(f.np, 2), false,
+        le = launch_persistent(c, k_linv_small<2>, 64, la, sizeof(float) * (size_t)linv_small_floats(f.np, 2), 0,
                                sh);
       } else {
         la.gstride = (linv_slot_floats(f.np, false) + 3) & ~3LL;
         const int64_t slots = std::min<int64_t>(f.count, c->num_sms);
         KSDF_CUDA(c, ensure(c->ws[WS_LINVSCR], sizeof(float) * (size_t)(la.gstride * slots + 4)));
         la.gscr = ptr<float>(c->ws[WS_LINVSCR]);
-        le = launch_persistent(c, k_linv<512, false, true>, 512, la, 0, true, sh);
+        le = launch_persistent(c, k_linv<512, false, true>, 512, la, 0, 1, sh);
       }
       KSDF_CUDA(c, le);
     }
@@ -1697,8 +1764,11 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
   return KSDF_OK;
 }
 
-// candidate size-class tables of the fit (largest class first; the first entry keeps its matrices in a
-// global slot).  Table 0 is the default; ksdf_autotune times them all on the model's own cells.  The result
+// candidate size-class tables of the fit: the fixed-point factorisation's classes, then the binary64 one's (largest
+// class first; `true` keeps the matrices in global slots).  Fixed point: one warp up to N = 95 (three rows per lane;
+// teams of two and three warps took 1.4 times as long at N = 64..80), then a warp per 32 rows; from N = 160 the global
+// slot with two teams of eight warps per SM beats shared memory with one team of seven (24.9 against 25.3 ms of fit at
+// 2M samples, 31.9 against 34.3 ms on cells of up to 512).  Table 0 is the default; ksdf_autotune times them all on the model's own cells.  The result
 // of a fit does not depend on the table (each cell's arithmetic is the same whatever the team size).
 ksdf_status device_math(ksdf_ctx* c, int fn, const double* x, int64_t n, double* y) {
   if (n > 0) launch(k_device_math, ceil_div(n, 256), 256, 0, c->stream, fn, x, n, y);
@@ -1706,29 +1776,41 @@ ksdf_status device_math(ksdf_ctx* c, int fn, const double* x, int64_t n, double*
   return KSDF_OK;
 }
 
-static const std::vector<std::vector<FitClassCfg>> kFitTables = {
-    // one warp up to 80, two up to 96, four up to 156, eight up to 218
-    {{kMaxNmax, 256, true}, {218, 256, false}, {156, 128, false}, {128, 128, false}, {96, 64, false},
-     {80, 32, false}, {64, 32, false}},
-    // one warp up to 96, two up to 128
-    {{kMaxNmax, 256, true}, {218, 256, false}, {156, 128, false}, {128, 64, false}, {96, 32, false},
-     {80, 32, false}, {64, 32, false}},
-    // one warp up to 64, two up to 128
-    {{kMaxNmax, 256, true}, {218, 256, false}, {156, 128, false}, {128, 64, false}, {96, 64, false},
-     {80, 64, false}, {64, 32, false}, {48, 32, false}},
-    // one warp up to 80, two up to 128, four up to 218
-    {{kMaxNmax, 256, true}, {218, 128, false}, {156, 128, false}, {128, 64, false}, {96, 64, false},
-     {80, 32, false}, {64, 32, false}},
-    // one warp up to 64, two up to 112, four up to 180, finer classes
-    {{kMaxNmax, 256, true}, {218, 256, false}, {180, 128, false}, {140, 128, false}, {112, 64, false},
-     {96, 64, false}, {80, 64, false}, {64, 32, false}},
-    // one warp up to 72, two up to 156, four up to 218
-    {{kMaxNmax, 256, true}, {218, 128, false}, {156, 64, false}, {128, 64, false}, {96, 64, false},
-     {72, 32, false}, {56, 32, false}, {40, 32, false}},
+static const std::vector<FitTable> kFitTables = {
+    {{{kMaxNmax, 512, true}, {256, 256, true}, {159, 160, false}, {127, 128, false}, {95, 32, false},
+      {79, 32, false}, {63, 32, false}},
+     // one warp up to 80, two up to 96, four up to 156, eight up to 218
+     {{kMaxNmax, 256, true}, {218, 256, false}, {156, 128, false}, {128, 128, false}, {96, 64, false},
+      {80, 32, false}, {64, 32, false}}},
+    {{{kMaxNmax, 512, true}, {256, 256, true}, {215, 224, false}, {159, 160, false}, {127, 128, false}, {95, 32, false},
+      {87, 32, false}, {71, 32, false}},
+     // one warp up to 96, two up to 128
+     {{kMaxNmax, 256, true}, {218, 256, false}, {156, 128, false}, {128, 64, false}, {96, 32, false},
+      {80, 32, false}, {64, 32, false}}},
+    {{{kMaxNmax, 512, true}, {256, 256, true}, {215, 224, false}, {159, 160, false}, {119, 128, false}, {95, 32, false},
+      {79, 32, false}, {47, 32, false}},
+     // one warp up to 64, two up to 128
+     {{kMaxNmax, 256, true}, {218, 256, false}, {156, 128, false}, {128, 64, false}, {96, 64, false},
+      {80, 64, false}, {64, 32, false}, {48, 32, false}}},
+    {{{kMaxNmax, 512, true}, {256, 256, true}, {215, 224, false}, {159, 160, false}, {127, 128, false}, {87, 32, false},
+      {79, 32, false}, {71, 32, false}},
+     // one warp up to 80, two up to 128, four up to 218
+     {{kMaxNmax, 256, true}, {218, 128, false}, {156, 128, false}, {128, 64, false}, {96, 64, false},
+      {80, 32, false}, {64, 32, false}}},
+    {{{kMaxNmax, 512, true}, {256, 256, true}, {215, 224, false}, {159, 160, false}, {127, 128, false}, {95, 32, false},
+      {79, 32, false}, {63, 32, false}},
+     // one warp up to 64, two up to 112, four up to 180, finer classes
+     {{kMaxNmax, 256, true}, {218, 256, false}, {180, 128, false}, {140, 128, false}, {112, 64, false},
+      {96, 64, false}, {80, 64, false}, {64, 32, false}}},
+    {{{kMaxNmax, 512, true}, {256, 256, true}, {183, 224, false}, {143, 160, false}, {119, 128, false}, {87, 32, false},
+      {71, 32, false}, {55, 32, false}},
+     // one warp up to 72, two up to 156, four up to 218
+     {{kMaxNmax, 256, true}, {218, 128, false}, {156, 64, false}, {128, 64, false}, {96, 64, false},
+      {72, 32, false}, {56, 32, false}, {40, 32, false}}},
 };
 
 int fit_table_count() { return (int)kFitTables.size(); }
-const std::vector<FitClassCfg>& fit_table(int i) { return kFitTables[(size_t)i]; }
+const FitTable& fit_table(int i) { return kFitTables[(size_t)i]; }
 
 // time every candidate table on the fitted model (each fit run twice, the second timed with CUDA events on
 // the context stream), keep the fastest in the context, and refit with it; the model is unchanged
@@ -1759,7 +1841,7 @@ ksdf_status autotune_fit(ksdf_ctx* c, int* chosen, double* ms) {
   double best_ms = 1e300;
   ksdf_status rs = KSDF_OK;
   for (int t = 0; t < fit_table_count() && rs == KSDF_OK; ++t) {
-    c->fit_cls = fit_table(t);
+    c->fit_tab = t;
     float tms = 0.f;
     for (int rep = 0; rep < 2 && rs == KSDF_OK; ++rep) {
       cudaEventRecord(e0, st);
@@ -1780,7 +1862,7 @@ ksdf_status autotune_fit(ksdf_ctx* c, int* chosen, double* ms) {
   cudaEventDestroy(e1);
   c->prof = prof;
   if (rs != KSDF_OK) return rs;
-  c->fit_cls = fit_table(best);
+  c->fit_tab = best;
   if (chosen) *chosen = best;
   rs = fit_model(c, ux, uv, un, S);
   return rs == KSDF_ERR_NOT_PD ? KSDF_OK : rs;

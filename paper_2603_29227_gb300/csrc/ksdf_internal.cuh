@@ -216,6 +216,10 @@ struct FitClassCfg {
   int np, team;
   bool gmat;
 };
+// the size classes (largest first) of the fixed-point factorisation and of the binary64 one
+struct FitTable {
+  std::vector<FitClassCfg> fx, f64;
+};
 }  // namespace ksdf
 
 struct ksdf_ctx {
@@ -228,10 +232,10 @@ struct ksdf_ctx {
   bool fitted = false;
   ksdf::Model m;
   ksdf::Model m_prev;  // the previous model during an update (its buffers are reused by the next one)
-  std::vector<ksdf::FitClassCfg> fit_cls;  // the fit's size classes (empty: the default table); ksdf_autotune
+  int fit_tab = 0;                         // the fit's size-class table; ksdf_autotune
   // workspaces
   ksdf::DevBuf status_word;       // uint32 device status
-  ksdf::DevBuf ws[32];            // general workspaces (grow only), indexed by role
+  ksdf::DevBuf ws[34];            // general workspaces (grow only), indexed by role
   int qt_chunks = 128;            // query tile shapes (ksdf_autotune_query): phase A's shared-memory budget in
   int qt_tc_small = 96;           // chunks of 8 samples, and the largest cell of phase B's 128-column TMEM class
   int64_t sched_max = 0;          // refit budget of ksdf_update (cells per update; 0 = every changed cell)
@@ -282,7 +286,7 @@ void prof_end(ksdf_ctx* c, cudaEvent_t a, const char* name);
 // ---- autotuning of the fit's size classes (ksdf_fit.cu) ----
 int fit_table_count();
 ksdf_status device_math(ksdf_ctx* c, int fn, const double* x, int64_t n, double* y);
-const std::vector<FitClassCfg>& fit_table(int i);
+const FitTable& fit_table(int i);
 ksdf_status autotune_fit(ksdf_ctx* c, int* chosen, double* ms);
 
 // ---- fork/join of the context stream with the auxiliary streams (ksdf_abi.cu) ----
@@ -350,13 +354,22 @@ enum WsRole {
   WS_UN = 28,
   WS_BRICK = 29,  // brick build: rank of each cell within its brick
   WS_SCHED = 30,  // refit scheduling: priority keys, cell ids, changed flags, previous ids
-  WS_BORD = 31    // query bins in coarse spatial order: coarse keys, ranks, order; bucket counts
+  WS_BORD = 31,   // query bins in coarse spatial order: coarse keys, ranks, order; bucket counts
+  WS_FIXSCR = 32,  // fixed-point fit scratch: global slots of the two largest classes
+  WS_FIXSCR2 = 33
 };
 constexpr int kQueryCounterCap = 10000;  // cap of the per-cell query counter (App. G)
 
 inline unsigned ceil_div(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 
 __host__ __device__ inline int64_t tri_sz(int64_t n) { return n * (n + 1) / 2; }
+// row of the packed lower-triangle entry t (t = i (i+1)/2 + j, j <= i)
+__device__ __forceinline__ int tri_row(int64_t t) {
+  int i = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+  while (tri_sz(i + 1) <= t) ++i;
+  while (tri_sz(i) > t) --i;
+  return i;
+}
 
 // cells up to this size run the variance contraction on the tensor cores (one MMA covers N <= 256)
 constexpr int kTcMaxN = 256;
