@@ -8,9 +8,8 @@
 // absolute rounding (2^-58 per entry of L, 2^-60 per sum) is below binary64's on these numbers: against 113-bit
 // arithmetic alpha's relative error is 0.5 to 0.9 of the binary64 factorisation's (geometric means over cells of the
 // benchmark scenes), L's is the same (both carry the kernel entries' rounding).
-// Measured (whole fit, kernel matrices to the last L^-1): 81,700 cells of mean N 80, 29.7 -> 22.5 ms; 865 cells of mean
-// N 473, 66.0 -> 31.9 ms (the FP32 L^-1 of N > 256 is half of that); a stream frame with a tenth of its cells at
-// N = 256, 35.0 -> 12.0 ms.  What bounds it now: the multiply-adds in the sums (about half of the pipe's rate, the
+// Measured (with the L^-1 kernels that run beside it): 81,700 cells of mean N 80, 29.3 -> 19.0 ms; 865 cells of mean N
+// 473, 48.6 -> 12.4 ms; a stream frame with a tenth of its cells at N = 256, 34.4 -> 8.3 ms.  What bounds it now: the multiply-adds in the sums (about half of the pipe's rate, the
 // panels' serial 8 x 8 blocks take the rest), with shared memory allowing five to nine cells per SM.
 //
 // Numbers.  "Q57 pair": v = h 2^27 + l with |l| <= 2^26 (two int32), value v 2^-57: L, y.  "Q60": int64, value 2^-60:
@@ -144,6 +143,11 @@ __device__ __forceinline__ void fx_write_l(const int2* Ls, int n8, int N, int t,
   }
 }
 
+// whether an entry of row N (t = its sum in Q60, v the entry) left the range |y_i| < 1, i.e. 2^-kFxYs
+__device__ __forceinline__ bool fx_y_out(long long t, int s2, int2 v) {
+  return (t >> (60 - s2)) != (t >> 63) || abs(v.x) >= 1 << (30 - kFxYs);
+}
+
 // One panel of a cell owned by one warp: a lane holds NS rows kb + lane + 32 s of the rows kb .. N (row N is the
 // right-hand side, ones times 2^-kFxYs, which becomes y).  The gather reads the panel rows' pairs once for all NS
 // rows; the pivots and the panel's multipliers go through shuffles, and all rows take the eight columns together.
@@ -217,7 +221,7 @@ __device__ __forceinline__ bool fx_panel(int2* Ls, const long long* A, int N, in
       for (int s = 0; s < NS; ++s) {
         v[s] = fx_scale(t[s], D, s2);
         if (kb + lane + 32 * s < n8 && (s > 0 || lane >= j)) Lp[j * cs + 32 * s] = v[s];
-        if (s == NS - 1 || s == NS - 2) bad |= kb + lane + 32 * s == N && (t[s] >> (58 - s2)) != (t[s] >> 63);
+        if (s == NS - 1) bad |= kb + lane + 32 * s == N && fx_y_out(t[s], s2, v[s]);
       }
 #pragma unroll
       for (int k = j + 1; k < 8; ++k) {
@@ -403,7 +407,7 @@ __global__ void __launch_bounds__(32 * W, W == 7 ? 1 : 16 / W) k_fit_fx(FixArgs 
             const int2 v = fx_scale(t, D, s2);
             if (lane >= j && i < n8) Lp[j * cs + lane] = v;
             if (GM && lane < 8) stage[8 * (kb + j) + lane] = v;
-            bad |= i == N && (t >> (58 - s2)) != (t >> 63);
+            bad |= i == N && fx_y_out(t, s2, v);
 #pragma unroll
             for (int k = j + 1; k < 8; ++k) {
               const int bh = __shfl_sync(FULL, v.x, k), bl = __shfl_sync(FULL, v.y, k);
@@ -433,7 +437,7 @@ __global__ void __launch_bounds__(32 * W, W == 7 ? 1 : 16 / W) k_fit_fx(FixArgs 
           const int s2 = s_e[j];
           const int2 v = fx_scale(t, s_d[j], s2);
           if (r < n8) Lp[j * cs + (r - kb)] = v;
-          bad |= r == N && (t >> (58 - s2)) != (t >> 63);
+          bad |= r == N && fx_y_out(t, s2, v);
 #pragma unroll
           for (int k = j + 1; k < 8; ++k) {
             const int2 b = GM ? stage[8 * (kb + j) + k] : Lp[j * cs + k];
