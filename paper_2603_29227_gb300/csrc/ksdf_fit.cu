@@ -949,16 +949,9 @@ __global__ void __launch_bounds__(TEAM, TEAM == 32 ? 12 : 256 / TEAM) k_fit(FitA
   }
 }
 
-// L^{-1} in FP32 for the variance contraction, one team per cell (persistent over cells order[first ..
-// first + count)).  L is rounded to FP32 (integer-bit conversion) into shared memory and each column of X =
-// L^{-1} is the forward substitution L x = e_j: X[j][j] = 1/L_jj and X[i][j] = -(sum_{k=j..i-1} L_ik X_kj) /
-// L_ii for i > j.  A lane owns a column and a warp a group of 32 consecutive columns, walking the rows
-// four at a time so that every X_kj load feeds four FFMAs; no synchronisation beyond the warp.
-//   INPLACE (one warp, small cells): the groups run in order and X overwrites L (a group only reads L in
-//     its own and later columns, and a row's L entries until that row is finished);
-//   otherwise one warp per group, all groups concurrently, each with its own buffer of (np - 32 g) rows.
-// The group's columns are then written in the 8-row blocked layout.  A separate kernel so that the fit's
-// warps keep the FP64 pipe busy; this one is FP32 only.
+// L^{-1} in FP32 for the variance contraction and the adjoint's solves.  L is rounded to FP32 (integer-bit
+// conversion) and each column of X = L^{-1} is the forward substitution L x = e_j: X[j][j] = 1/L_jj and X[i][j] =
+// -(sum_{k=j..i-1} L_ik X_kj) / L_ii for i > j.  Separate kernels from the factorisation's, FP32 only.
 struct LinvArgs {
   const uint32_t* order;
   int64_t first, count;
@@ -970,19 +963,9 @@ struct LinvArgs {
   float* linv32;
   const int64_t* ltc_off;
   float* ltc;       // the cell's image at ltc + ltc_off[g]
-  float* gscr;      // per-CTA global slot (largest class): linv_slot_floats(np, false)
-  int64_t gstride;
   int np;
   int* counter;
 };
-
-// float offset of group g's buffer (after the reciprocal diagonal and L) and the slot size
-__host__ __device__ inline int64_t linv_group_off(int np, int g) {
-  return (((int64_t)np + 3) & ~3LL) + tri_sz(np) + 32LL * ((int64_t)g * np - 32LL * tri_sz(g - 1));
-}
-__host__ __device__ inline int64_t linv_slot_floats(int np, bool inplace) {
-  return inplace ? (((int64_t)np + 3) & ~3LL) + tri_sz(np) : linv_group_off(np, (np + 31) / 32);
-}
 
 // L^{-1} of the cells with N <= 256, a CTA of W warps per cell (persistent).  Shared memory holds L in FP32
 // with every row padded to a multiple of four floats (row i at lrow_off(i)), the reciprocal diagonal, and per
@@ -1119,7 +1102,7 @@ __global__ void __launch_bounds__(32 * W) k_linv_small(LinvArgs a) {
       }
       // tensor-core image: quads of this group's columns, all Np rows (FP32; the query splits it into TF32
       // hi and lo parts in shared memory)
-      if (N <= kTcMaxN) {
+      {
         const int np16 = tc_np(N);
         const int q1 = min(base + 32, tc_kp(N)) >> 2;
         float* img = a.ltc + a.ltc_off[g];
@@ -1142,121 +1125,139 @@ __global__ void __launch_bounds__(32 * W) k_linv_small(LinvArgs a) {
   }
 }
 
-template <int TEAM, bool INPLACE, bool GMAT>
-__global__ void __launch_bounds__(TEAM) k_linv(LinvArgs a) {
+// L^{-1} of larger cells (classes above 128): a CTA of four warps per (cell, group of 32 columns) -- the groups are independent,
+// so a cell spreads over many CTAs.  The group's X = L^{-1} columns live in shared memory; the rows advance in blocks
+// of 32: the block's rows of L come in (binary64 -> FP32, 128 columns at a time), the CTA forms C = L[block, base..) X
+// for the finished rows (a thread four rows x two columns: eight 16- and 8-byte loads feed 32 FFMAs), one warp solves
+// the 32 x 32 triangle
+// (a lane per column), and the block is written in both layouts.  Every entry is the same sum in the same order
+// (ascending k) as in k_linv_small.
+// Measured: 865 cells of mean N 473, 15.7 -> 3.8 ms (one CTA of 16 warps per cell on a global slot before); latency of
+// the row blocks' chain bounds it.  Classes up to 128 stay on k_linv_small (0.84 ms for 7,400 cells of N 96..127).
+constexpr int kLbThreads = 128;
+constexpr int kLbChunk = 128;
+__host__ __device__ inline size_t linv_big_smem(int np) {
+  return sizeof(float) * (32 * (size_t)(kLbChunk + 4) + 32 * (size_t)((np + 31) & ~31) + 32 * 33 + 32);
+}
+
+__global__ void __launch_bounds__(kLbThreads) k_linv_big(LinvArgs a) {
   extern __shared__ __align__(16) float smf[];
-  __shared__ int s_cell;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int np = a.np;
-  float* ws = GMAT ? a.gscr + (int64_t)blockIdx.x * a.gstride : smf;
-  float* dg = ws;
-  float* L = ws + ((np + 3) & ~3);
+  __shared__ int s_item;
+  const int tid = threadIdx.x, lane = tid & 31;
+  constexpr int ls = kLbChunk + 4;
+  float* Lt = smf;                              // [32][ls]: the block's rows, a chunk of columns
+  float* X = Lt + 32 * ls;                      // [row - base][32]
+  float* C = X + 32 * ((a.np + 31) & ~31);      // [32][33]
+  float* dg = C + 32 * 33;                      // [32]
+  const int ngr = (a.np + 31) >> 5;
   for (;;) {
-    if (tid == 0) {
-      const int w = atomicAdd(a.counter, 1);
-      s_cell = w < a.count ? (int)a.order[a.first + w] : -1;
-    }
-    fit_sync(TEAM);
-    const int g = s_cell;
-    if (g < 0) break;
-    const int N = a.n32[g];
-    if (N == 0 || a.status[g] != KSDF_CELL_OK) {
-      fit_sync(TEAM);
+    if (tid == 0) s_item = atomicAdd(a.counter, 1);
+    __syncthreads();
+    const int item = s_item;
+    if (item >= a.count * ngr) break;
+    const int g = (int)a.order[a.first + item / ngr];
+    const int N = a.n32[g], base = 32 * (item % ngr);
+    if (base >= N || a.status[g] != KSDF_CELL_OK) {
+      __syncthreads();
       continue;
     }
-    const int64_t T = tri_sz(N);
     const double* Ld = a.chol64 + a.chol_off[g];
-    for (int64_t e0 = tid; e0 < T; e0 += 8 * (int64_t)TEAM) {  // eight loads in flight per thread
-      double v[8];
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        const int64_t e = e0 + (int64_t)r * TEAM;
-        v[r] = e < T ? Ld[e] : 0.0;
-      }
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        const int64_t e = e0 + (int64_t)r * TEAM;
-        if (e < T) L[e] = d2f_bits(v[r]);
-      }
-    }
-    fit_sync(TEAM);
-    for (int j = tid; j < N; j += TEAM) dg[j] = 1.f / L[tri_sz(j) + j];
-    fit_sync(TEAM);
     float* Iout = a.linv32 + a.linv_off[g];
-    const int nR = (N + 7) >> 3;
-    for (int gi = INPLACE ? 0 : warp; 32 * gi < N; gi += INPLACE ? 1 : TEAM / 32) {
-      const int base = 32 * gi, j = base + lane;
-      // X[k][j] lives at xs[k * ldx] (in place: L's packed row k; else the group's buffer)
-      float* xcol = INPLACE ? L + j : ws + linv_group_off(np, gi) - (int64_t)base * 32 + lane;
-      for (int i0 = base; i0 < N; i0 += 4) {
-        const float* L0 = L + tri_sz(i0);
-        const float* L1 = L + tri_sz(min(i0 + 1, N - 1));
-        const float* L2 = L + tri_sz(min(i0 + 2, N - 1));
-        const float* L3 = L + tri_sz(min(i0 + 3, N - 1));
-        float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f;
-#pragma unroll 4
-        for (int k = base; k < i0; ++k) {
-          float x;
-          if (INPLACE) x = k >= j ? xcol[tri_sz(k)] : 0.f;  // X[k][j], zero above the diagonal
-          else x = xcol[(int64_t)k * 32];
-          c0 = fmaf(L0[k], x, c0);
-          c1 = fmaf(L1[k], x, c1);
-          c2 = fmaf(L2[k], x, c2);
-          c3 = fmaf(L3[k], x, c3);
-        }
-        float xv[4];
-        xv[0] = i0 > j ? -c0 * dg[i0] : (i0 == j ? dg[j] : 0.f);
-        if (i0 + 1 < N) {
-          c1 = fmaf(L1[i0], xv[0], c1);
-          xv[1] = i0 + 1 > j ? -c1 * dg[i0 + 1] : (i0 + 1 == j ? dg[j] : 0.f);
-          if (i0 + 2 < N) {
-            c2 = fmaf(L2[i0 + 1], xv[1], fmaf(L2[i0], xv[0], c2));
-            xv[2] = i0 + 2 > j ? -c2 * dg[i0 + 2] : (i0 + 2 == j ? dg[j] : 0.f);
-            if (i0 + 3 < N) {
-              c3 = fmaf(L3[i0 + 2], xv[2], fmaf(L3[i0 + 1], xv[1], fmaf(L3[i0], xv[0], c3)));
-              xv[3] = i0 + 3 > j ? -c3 * dg[i0 + 3] : (i0 + 3 == j ? dg[j] : 0.f);
-            }
+    const int nR = (N + 7) >> 3, np16 = tc_np(N);
+    float* img = a.ltc + a.ltc_off[g];
+    for (int i0 = base; i0 < N; i0 += 32) {
+      const int kb = i0 - base;  // finished rows of X
+      const int r0 = 4 * (tid >> 4), c0 = 2 * (tid & 15);
+      float c[4][2] = {};
+      for (int k0 = 0; k0 <= kb; k0 += kLbChunk) {
+        // the block's rows of L, columns base + k0 .. (zero beyond the diagonal and past row N - 1); the last chunk
+        // ends with the block's own columns
+        const int kw = min(kLbChunk, kb + 32 - k0);
+        constexpr int RW = 32 / (kLbThreads / 32);  // rows of a warp: all their loads in flight
+        double v[RW][kLbChunk / 32];
+        const int wr = (tid >> 5) * RW;
+#pragma unroll
+        for (int r = 0; r < RW; ++r) {
+          const int i = i0 + wr + r;
+          const double* Li = Ld + tri_sz(i) + base + k0;
+#pragma unroll
+          for (int u = 0; u < kLbChunk / 32; ++u) {
+            const int k = lane + 32 * u;
+            v[r][u] = k < kw && i < N && base + k0 + k <= i ? Li[k] : 0.0;
           }
         }
-        // rows i0.. are finished: store (in place: only on or below the diagonal and inside the matrix)
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
+        for (int r = 0; r < RW; ++r)
+#pragma unroll
+          for (int u = 0; u < kLbChunk / 32; ++u)
+            if (lane + 32 * u < kw) Lt[(wr + r) * ls + lane + 32 * u] = d2f_bits(v[r][u]);
+        __syncthreads();
+        const float* Lr = Lt + r0 * ls;
+        const float* Xk = X + k0 * 32 + c0;
+        const int ke = min(kLbChunk, kb - k0);
+#pragma unroll 2
+        for (int k = 0; k < ke; k += 4) {
+          float4 l[4];
+          float2 x[4];
+#pragma unroll
+          for (int r = 0; r < 4; ++r) l[r] = *reinterpret_cast<const float4*>(Lr + r * ls + k);
+#pragma unroll
+          for (int u = 0; u < 4; ++u) x[u] = *reinterpret_cast<const float2*>(Xk + (k + u) * 32);
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            c[r][0] = fmaf(l[r].x, x[0].x, c[r][0]);
+            c[r][1] = fmaf(l[r].x, x[0].y, c[r][1]);
+            c[r][0] = fmaf(l[r].y, x[1].x, c[r][0]);
+            c[r][1] = fmaf(l[r].y, x[1].y, c[r][1]);
+            c[r][0] = fmaf(l[r].z, x[2].x, c[r][0]);
+            c[r][1] = fmaf(l[r].z, x[2].y, c[r][1]);
+            c[r][0] = fmaf(l[r].w, x[3].x, c[r][0]);
+            c[r][1] = fmaf(l[r].w, x[3].y, c[r][1]);
+          }
+        }
+        if (k0 + kLbChunk <= kb) __syncthreads();  // the tile is read before the next chunk comes in
+      }
+      const int kd = kb & (kLbChunk - 1);  // the block's own columns in the last chunk
+      if (tid < 32) dg[tid] = i0 + tid < N ? 1.f / Lt[tid * ls + kd + tid] : 0.f;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        C[(r0 + r) * 33 + c0] = c[r][0];
+        C[(r0 + r) * 33 + c0 + 1] = c[r][1];
+      }
+      __syncthreads();
+      if (tid < 32) {
+        const int j = base + lane;  // the lane's column
+        float x[32];
+#pragma unroll
+        for (int r = 0; r < 32; ++r) {
+          float c = C[r * 33 + lane];
+          const float* Lr = Lt + r * ls + kd;
+#pragma unroll
+          for (int s = 0; s < 32; ++s)
+            if (s < r) c = fmaf(Lr[s], x[s], c);
           const int i = i0 + r;
-          if (i < N) {
-            if (INPLACE) {
-              if (j <= i) xcol[tri_sz(i)] = xv[r];
-            } else {
-              xcol[(int64_t)i * 32] = xv[r];
-            }
-          }
-        }
-        if (INPLACE) __syncwarp();  // rows of L read by other lanes' columns are overwritten in place
-      }
-      // blocked output of the group's columns (columns N .. 8 nR - 1 of the last block are zero)
-      if (j < 8 * nR) {
-        for (int R = j >> 3; R < nR; ++R) {
-          float v[8];
-#pragma unroll
-          for (int r = 0; r < 8; ++r) {
-            const int i = 8 * R + r;
-            v[r] = (j < N && i < N && i >= j) ? (INPLACE ? xcol[tri_sz(i)] : xcol[(int64_t)i * 32]) : 0.f;
-          }
-          float4* dst = reinterpret_cast<float4*>(Iout + linv_block_off(R) + (int64_t)j * 8);
-          dst[0] = make_float4(v[0], v[1], v[2], v[3]);
-          dst[1] = make_float4(v[4], v[5], v[6], v[7]);
+          x[r] = i < N && j < N ? (i > j ? -c * dg[r] : (i == j ? dg[r] : 0.f)) : 0.f;
+          X[(kb + r) * 32 + lane] = x[r];
         }
       }
-      // the tensor-core image (column j of L^-1 is K index j of the B operand): all Np rows, zero padded, FP32
-      if (N <= kTcMaxN && j < tc_kp(N)) {
-        const int np16 = tc_np(N);
-        float* col = a.ltc + a.ltc_off[g] + (int64_t)(j >> 2) * np16 * 4 + (j & 3);
-        for (int i = 0; i < np16; ++i)
-          col[(int64_t)i * 4] =
-              (j < N && i < N && i >= j) ? (INPLACE ? xcol[tri_sz(i)] : xcol[(int64_t)i * 32]) : 0.f;
+      __syncthreads();
+      // out: 8-row blocks (a column's 8 rows contiguous, 32 columns 1 KB) and the tensor-core image's quads
+      for (int e = tid; e < 4 * 32 * 2; e += kLbThreads) {
+        const int R = (i0 >> 3) + (e >> 6), col = (e >> 1) & 31, h = e & 1;
+        if (R < nR && base + col < 8 * R + 8) {
+          const float* xs = X + (8 * R + 4 * h - base) * 32 + col;
+          reinterpret_cast<float4*>(Iout + linv_block_off(R) + (int64_t)(base + col) * 8)[h] =
+              make_float4(xs[0], xs[32], xs[64], xs[96]);
+        }
       }
-      if (INPLACE) __syncwarp();
+      for (int e = tid; N <= kTcMaxN && e < 8 * 32; e += kLbThreads) {
+        const int q = e >> 5, i = i0 + (e & 31);
+        if (i < np16 && base + 4 * q < tc_kp(N))
+          *reinterpret_cast<float4*>(img + ((int64_t)((base >> 2) + q) * np16 + i) * 4) =
+              *reinterpret_cast<const float4*>(X + (i - base) * 32 + 4 * q);
+      }
     }
-    fit_sync(TEAM);
+    __syncthreads();
   }
 }
 
@@ -1662,21 +1663,22 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
       la.linv32 = ptr<float>(m.linv32);
       la.ltc_off = ptr<int64_t>(m.ltc_off);
       la.ltc = ptr<float>(m.ltc);
-      la.gscr = nullptr;
-      la.gstride = 0;
       la.np = f.np;
       if (f.np <= 96) {
         le = launch_persistent(c, k_linv_small<1>, 32, la, sizeof(float) * (size_t)linv_small_floats(f.np, 1), 0,
                                sh);
-      } else if (f.np <= kTcMaxN) {
+      } else if (f.np <= 128) {
         le = launch_persistent(c, k_linv_small<2>, 64, la, sizeof(float) * (size_t)linv_small_floats(f.np, 2), 0,
                                sh);
       } else {
-        la.gstride = (linv_slot_floats(f.np, false) + 3) & ~3LL;
-        const int64_t slots = std::min<int64_t>(f.count, c->num_sms);
-        KSDF_CUDA(c, ensure(c->ws[WS_LINVSCR], sizeof(float) * (size_t)(la.gstride * slots + 4)));
-        la.gscr = ptr<float>(c->ws[WS_LINVSCR]);
-        le = launch_persistent(c, k_linv<512, false, true>, 512, la, 0, 1, sh);
+        // (the class's np may exceed its largest cell: groups beyond a cell's N end at once)
+        const size_t lsm = linv_big_smem(f.np);
+        KSDF_CUDA(c, cudaFuncSetAttribute(k_linv_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lsm));
+        int occ = 0;
+        KSDF_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_linv_big, kLbThreads, lsm));
+        const int64_t items = f.count * ((f.np + 31) / 32);
+        launch(k_linv_big, (unsigned)std::min<int64_t>(items, (int64_t)std::max(1, occ) * c->num_sms), kLbThreads, lsm,
+               sh, la);
       }
       KSDF_CUDA(c, le);
     }
@@ -1767,8 +1769,8 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
 // candidate size-class tables of the fit: the fixed-point factorisation's classes, then the binary64 one's (largest
 // class first; `true` keeps the matrices in global slots).  Fixed point: one warp up to N = 95 (three rows per lane;
 // teams of two and three warps took 1.4 times as long at N = 64..80), then a warp per 32 rows; from N = 160 the global
-// slot with two teams of eight warps per SM beats shared memory with one team of seven (24.9 against 25.3 ms of fit at
-// 2M samples, 31.9 against 34.3 ms on cells of up to 512).  Table 0 is the default; ksdf_autotune times them all on the model's own cells.  The result
+// slot with two teams of eight warps per SM beats shared memory with one team of seven (24.1 against 24.8 ms of fit at
+// 2M samples, 19.8 against 20.7 ms on cells of up to 512).  Table 0 is the default; ksdf_autotune times them all on the model's own cells.  The result
 // of a fit does not depend on the table (each cell's arithmetic is the same whatever the team size).
 ksdf_status device_math(ksdf_ctx* c, int fn, const double* x, int64_t n, double* y) {
   if (n > 0) launch(k_device_math, ceil_div(n, 256), 256, 0, c->stream, fn, x, n, y);

@@ -347,7 +347,6 @@ enum WsRole {
   WS_CELLQ = 21,  // per cell query counts / offsets
   WS_FITSCR = 22, // FP64 fit scratch
   WS_BW = 23,     // backward accumulators
-  WS_LINVSCR = 24, // FP32 L^-1 scratch of the largest cells
   WS_TOUCH = 25,  // update: per cell touched flag and previous id
   WS_UX = 26,     // update: the union of old and new samples (positions, variances, normals)
   WS_UV = 27,
