@@ -15,6 +15,7 @@
 // Kernel 1 recomputes k' per (query, winner) tile and accumulates alpha_bar / X_bar per sample; kernel 2 runs
 // once per touched cell.
 #include "ksdf_internal.cuh"
+#include "ksdf_small.cuh"
 
 #include <algorithm>
 
@@ -72,6 +73,38 @@ __global__ void k_bw_tiles(const int64_t* cnt, const int64_t* off, const int64_t
 __global__ void k_ntiles_w(const int64_t* cnt, int64_t n, int64_t* nt) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) nt[i] = (cnt[i] + kTW - 1) / kTW;
+}
+
+// the same for a small batch in one CTA (ksdf_small.cuh); cnt holds zeros on entry
+__global__ void __launch_bounds__(kSmallThreads) k_bw_group_small(const int32_t* winner, int Q, int64_t G, int64_t* cnt,
+                                                                  float* d_xq, int dim, int32_t* sorted, int4* tiles,
+                                                                  int64_t* tot, uint32_t* st) {
+  __shared__ SmallSort s;
+  for (int q = threadIdx.x; q < Q; q += kSmallThreads) {
+    int w = winner[q];
+    if (w >= G) {
+      atomicOr(st, ST_CAPACITY);
+      w = -1;
+    }
+    if (w < 0)
+      for (int j = 0; j < dim; ++j) d_xq[(int64_t)q * dim + j] = 0.f;
+    s.key[q] = w < 0 ? kEmptyKey : (uint64_t)w;
+    s.idx[q] = q;
+  }
+  int gid[2];
+  const int ng = small_group(s, Q, gid);
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int i = 2 * threadIdx.x + u;
+    if (i < Q) sorted[i] = s.idx[i];
+  }
+  const int nt = small_tiles(s, ng, kTW, [&](int g, int t0, int n) {
+    const int b = s.start[g], c = s.start[g + 1] - b;
+    const int w = (int)s.key[b];
+    cnt[w] = c;
+    for (int t = 0; t < n; ++t) tiles[t0 + t] = make_int4(w, b + t * kTW, min(c - t * kTW, kTW), 0);
+  });
+  if (threadIdx.x < 4) tot[threadIdx.x] = threadIdx.x == 0 ? nt : 0;
 }
 
 struct BwArgs {
@@ -499,14 +532,18 @@ ksdf_status run_backward(ksdf_ctx* c, const float* xq, int64_t Q, const int8_t* 
   double* abar = ptr<double>(c->ws[WS_BW]);
   cudaEvent_t e_b = prof_begin(c), e0 = prof_begin(c);
   KSDF_CUDA(c, cudaMemsetAsync(cnt, 0, sizeof(int64_t) * G, st));
-  KSDF_CUDA(c, cudaMemsetAsync(tot, 0, sizeof(int64_t) * 4, st));
   KSDF_CUDA(c, cudaMemsetAsync(abar, 0, sizeof(double) * (m.M + 1), st));
-  launch(k_bw_count, ceil_div(Q, 256), 256, 0, st, winner, Q, G, rank, cnt, d_xq, p.dim, stw);
-  KSDF_CUDA(c, scan_i64(cnt, off, G, nullptr, c->ws[WS_SCAN], st));
-  launch(k_ntiles_w, ceil_div(G, 256), 256, 0, st, cnt, G, nt);
-  KSDF_CUDA(c, scan_i64(nt, toff, G, &tot[0], c->ws[WS_SCAN], st));
-  launch(k_bw_scatter, ceil_div(Q, 256), 256, 0, st, winner, rank, Q, G, off, sorted);
-  launch(k_bw_tiles, ceil_div(G, 256), 256, 0, st, cnt, off, toff, G, tiles);
+  if (Q <= kSmallQ) {
+    launch(k_bw_group_small, 1, kSmallThreads, 0, st, winner, (int)Q, G, cnt, d_xq, p.dim, sorted, tiles, tot, stw);
+  } else {
+    KSDF_CUDA(c, cudaMemsetAsync(tot, 0, sizeof(int64_t) * 4, st));
+    launch(k_bw_count, ceil_div(Q, 256), 256, 0, st, winner, Q, G, rank, cnt, d_xq, p.dim, stw);
+    KSDF_CUDA(c, scan_i64(cnt, off, G, nullptr, c->ws[WS_SCAN], st));
+    launch(k_ntiles_w, ceil_div(G, 256), 256, 0, st, cnt, G, nt);
+    KSDF_CUDA(c, scan_i64(nt, toff, G, &tot[0], c->ws[WS_SCAN], st));
+    launch(k_bw_scatter, ceil_div(Q, 256), 256, 0, st, winner, rank, Q, G, off, sorted);
+    launch(k_bw_tiles, ceil_div(G, 256), 256, 0, st, cnt, off, toff, G, tiles);
+  }
   prof_end(c, e0, "backward.group");
   BwArgs a;
   a.tiles = tiles;
