@@ -378,81 +378,149 @@ __global__ void __launch_bounds__(kTQ) k_bw_query(BwArgs a, const float* xq, Par
   }
 }
 
-// per touched cell: b = A^{-1} alpha_bar.  b0 = L^{-T} L^{-1} alpha_bar with the FP32 L^{-1}; one step of
+// Per touched cell: b = A^{-1} alpha_bar.  b0 = L^{-T} L^{-1} alpha_bar with the FP32 L^{-1}; one step of
 // iterative refinement against the FP64 factor, r = alpha_bar - L (L^T b0) (the only FP64 work, N^2
 // FMAs), b = b0 + L^{-T} L^{-1} r; then the alpha-path X_bar terms in FP32.
-__device__ void linv_solve32(const float* Lb, int n, const float* rhs, float* y, float* out, bool add) {
+//
+// Every step is a chain of dependent loads and FMAs per thread.  With many cells touched the SM hides it behind other
+// cells: 64 threads a cell and little shared memory, the factors read through the caches (cells above kBwSplitN apart,
+// so that the others are not charged their shared memory).  A small batch (kSmallQ) touches a few dozen cells and
+// waits for the slowest: 128 threads a cell, both factors copied to shared memory first with all loads in flight, up
+// to kBwSmemN samples (copying in the large batches too took 8.9 instead of 3.9 ms for 61,000 cells: four to seven
+// cells per SM in place of 32), and 256 threads above.  The terms through alpha take two samples per packed instruction.
+// Measured: 61,000 cells 3.85 -> 2.80 ms, 512 queries' cells 151 -> 58 us.  Bound by load latency, the FP64 pipe at 36%.
+constexpr int kBwSplitN = 128;
+constexpr int kBwSmemN = 160;
+// shared memory: [n] alpha_bar, [n] t, [n] b0 (double) | [n] rhs, [n] y, [n] b, then the samples' x, y, z, alpha
+// (floats), n rounded up to 4 | staged: L^{-1} | L (double)
+__host__ __device__ inline size_t bw_vec_bytes(int n) { return (size_t)52 * ((n + 3) & ~3); }
+__host__ __device__ inline size_t bw_smem_bytes(int n, bool staged) {
+  return bw_vec_bytes(n) + (staged ? 4 * (size_t)linv_blocked_size(n) + 8 * (size_t)tri_sz(n) : 0);
+}
+
+// the cells with queries in two lists of G ints, those of at most `bound` samples and the larger ones; cnt their lengths
+__global__ void k_bw_cells(const int64_t* qcnt, const int32_t* cell_n, int64_t G, int bound, int32_t* list, int* cnt) {
+  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const bool hit = g < G && qcnt[g] != 0;
+  const int cl = hit ? (cell_n[g] <= bound ? 0 : 1) : -1;
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const unsigned m = __ballot_sync(0xffffffffu, cl == c);
+    if (m == 0) continue;
+    int base = 0;
+    if (lane == 0) base = atomicAdd(&cnt[c], __popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (cl == c) list[c * G + base + __popc(m & ((1u << lane) - 1u))] = (int32_t)g;
+  }
+}
+
+template <int NT>
+__device__ __forceinline__ void linv_solve32(const float* Lb, int n, const float* rhs, float* y, float* out, bool add) {
   // y = L^{-1} rhs (rows over threads; 8 consecutive rows share a 32-byte sector per column)
-  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+  for (int j = threadIdx.x; j < n; j += NT) {
     const float* row = Lb + linv_block_off(j >> 3) + (j & 7);
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;  // four independent chains
     int i = 0;
+#pragma unroll 2
     for (; i + 3 <= j; i += 4) {
-      a0 = fmaf(row[(int64_t)i * 8], rhs[i], a0);
-      a1 = fmaf(row[(int64_t)(i + 1) * 8], rhs[i + 1], a1);
-      a2 = fmaf(row[(int64_t)(i + 2) * 8], rhs[i + 2], a2);
-      a3 = fmaf(row[(int64_t)(i + 3) * 8], rhs[i + 3], a3);
+      a0 = fmaf(row[i * 8], rhs[i], a0);
+      a1 = fmaf(row[(i + 1) * 8], rhs[i + 1], a1);
+      a2 = fmaf(row[(i + 2) * 8], rhs[i + 2], a2);
+      a3 = fmaf(row[(i + 3) * 8], rhs[i + 3], a3);
     }
-    for (; i <= j; ++i) a0 = fmaf(row[(int64_t)i * 8], rhs[i], a0);
+    for (; i <= j; ++i) a0 = fmaf(row[i * 8], rhs[i], a0);
     y[j] = (a0 + a1) + (a2 + a3);
   }
   __syncthreads();
   // out (+)= L^{-T} y (columns over threads; the 8 rows of a block at one column are contiguous)
   const int nb = (n + 7) >> 3;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+  for (int i = threadIdx.x; i < n; i += NT) {
     float acc = 0.f;
+#pragma unroll 2
     for (int R = i >> 3; R < nb; ++R) {
-      const float4* v = reinterpret_cast<const float4*>(Lb + linv_block_off(R) + (int64_t)i * 8);
-      const float4 l0 = __ldg(v), l1 = __ldg(v + 1);
+      const float4* v = reinterpret_cast<const float4*>(Lb + linv_block_off(R) + i * 8);
+      const float4 l0 = v[0], l1 = v[1];
       const float* yy = y + 8 * R;
       const int rmax = min(8, n - 8 * R);
       const float lr[8] = {l0.x, l0.y, l0.z, l0.w, l1.x, l1.y, l1.z, l1.w};
-      for (int r = 0; r < rmax; ++r) acc = fmaf(lr[r], yy[r], acc);
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+        if (r < rmax) acc = fmaf(lr[r], yy[r], acc);
     }
     out[i] = add ? out[i] + acc : acc;
   }
   __syncthreads();
 }
 
-constexpr int kBwCellThreads = 64;  // two warps per cell: ~70-row cells keep most lanes busy, 32 cells per SM
-constexpr int kBwCellSmallN = 128;  // the small-cell launch: shared memory for at most this many samples
+struct BwCellArgs {
+  const int32_t* list;  // the class's cells
+  const int* count;
+  const int64_t* ts_off;
+  const int32_t* cell_n;
+  const int64_t* chol_off;
+  const double* chol64;
+  const int64_t* linv_off;
+  const float* linv32;
+  const float4* mf4;
+  const int32_t* mgid;
+  const double* abar;
+  float* d_x;
+};
 
-template <bool MATERN>
-__global__ void __launch_bounds__(kBwCellThreads) k_bw_cell(const int64_t* qcnt, int64_t G, const int64_t* ts_off,
-                                                 const int32_t* cell_n, const int64_t* chol_off, const double* chol64,
-                                                 const int64_t* linv_off, const float* linv32, const float4* mf4,
-                                                 const int32_t* mgid, const double* abar, Params p, float* d_x,
-                                                 int nlo, int nhi) {
-  extern __shared__ double sh[];  // [n] alpha_bar, [n] t, [n] b0 (double), then floats: rhs, y, b
-  for (int64_t g = blockIdx.x; g < G; g += gridDim.x) {
-    if (qcnt[g] == 0) continue;
-    const int n = cell_n[g];
-    if (n < nlo || n > nhi) continue;  // another launch's size class
-    const int64_t m0 = ts_off[g];
-    const double* L = chol64 + chol_off[g];
-    const float* Lb = linv32 + linv_off[g];
-    double* sa = sh;
-    double* st = sh + n;
-    double* sbd = sh + 2 * n;
-    float* srhs = reinterpret_cast<float*>(sh + 3 * n);
-    float* sy = srhs + n;
-    float* sb = sy + n;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      sa[i] = abar[m0 + i];
+template <bool MATERN, bool SM, int NT>
+__global__ void __launch_bounds__(NT) k_bw_cell(BwCellArgs a, Params p) {
+  extern __shared__ __align__(16) unsigned char bwsm[];
+  const int tid = threadIdx.x;
+  const int count = *a.count;
+  for (int e = blockIdx.x; e < count; e += gridDim.x) {
+    const int g = a.list[e];
+    const int n = a.cell_n[g], n4 = (n + 3) & ~3;
+    const int64_t m0 = a.ts_off[g];
+    double* sa = reinterpret_cast<double*>(bwsm);
+    double* st = sa + n4;
+    double* sbd = st + n4;
+    float* srhs = reinterpret_cast<float*>(sbd + n4);
+    float* sy = srhs + n4;
+    float* sb = sy + n4;
+    float* sx = sb + n4;  // x, y, z, alpha, n4 each
+    const float* Lb = a.linv32 + a.linv_off[g];
+    const double* L = a.chol64 + a.chol_off[g];
+    if (SM) {
+      float4* sl = reinterpret_cast<float4*>(bwsm + bw_vec_bytes(n));
+      const int nl = (int)(linv_blocked_size(n) >> 2), T = (int)tri_sz(n);
+      double* sd = reinterpret_cast<double*>(sl + nl);
+      const float4* src = reinterpret_cast<const float4*>(Lb);
+#pragma unroll 8
+      for (int i = tid; i < nl; i += NT) sl[i] = src[i];
+#pragma unroll 8
+      for (int i = tid; i < T; i += NT) sd[i] = L[i];
+      Lb = reinterpret_cast<const float*>(sl);
+      L = sd;
+    }
+    for (int i = tid; i < n4; i += NT) {
+      const float4 v = i < n ? a.mf4[m0 + i] : make_float4(0.f, 0.f, 0.f, 0.f);  // (padding: zero weight)
+      sx[i] = v.x;
+      sx[n4 + i] = v.y;
+      sx[2 * n4 + i] = v.z;
+      sx[3 * n4 + i] = v.w;
+      if (i >= n) sb[i] = 0.f;
+    }
+    for (int i = tid; i < n; i += NT) {
+      sa[i] = a.abar[m0 + i];
       srhs[i] = (float)sa[i];
     }
     __syncthreads();
-    linv_solve32(Lb, n, srhs, sy, sb, false);  // b0
-    for (int i = threadIdx.x; i < n; i += blockDim.x) sbd[i] = (double)sb[i];  // converted once, not per FMA
+    linv_solve32<NT>(Lb, n, srhs, sy, sb, false);  // b0
+    for (int i = tid; i < n; i += NT) sbd[i] = (double)sb[i];  // converted once, not per FMA
     __syncthreads();
     // t = L^T b0: rows in lockstep, threads over columns k (coalesced row reads)
-    for (int k = threadIdx.x; k < n; k += blockDim.x) st[k] = 0.0;
-    for (int k0 = 0; k0 < n; k0 += blockDim.x) {
-      const int k = k0 + threadIdx.x;
+    for (int k0 = 0; k0 < n; k0 += NT) {
+      const int k = k0 + tid;
       double c0 = 0.0, c1 = 0.0, c2 = 0.0, c3 = 0.0;  // four independent chains (DFMA latency ~64 cycles)
       // a warp walks rows from its first lane's column so that a row's loads coalesce; entries above the
       // diagonal (k > i, read in bounds from the following row) are masked to zero
-      int i = k0 + (threadIdx.x & ~31);
+      int i = k0 + (tid & ~31);
       if (k < n) {
         for (; i + 3 < n; i += 4) {
           c0 = fma(k <= i ? L[tri_sz(i) + k] : 0.0, sbd[i], c0);
@@ -466,8 +534,8 @@ __global__ void __launch_bounds__(kBwCellThreads) k_bw_cell(const int64_t* qcnt,
     }
     __syncthreads();
     // r = alpha_bar - L t (rows over threads)
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const double* Li = L + (int64_t)i * (i + 1) / 2;
+    for (int i = tid; i < n; i += NT) {
+      const double* Li = L + tri_sz(i);
       double c0 = sa[i], c1 = 0.0, c2 = 0.0, c3 = 0.0;
       int k = 0;
       for (; k + 3 <= i; k += 4) {
@@ -480,29 +548,38 @@ __global__ void __launch_bounds__(kBwCellThreads) k_bw_cell(const int64_t* qcnt,
       srhs[i] = (float)((c0 + c1) + (c2 + c3));
     }
     __syncthreads();
-    linv_solve32(Lb, n, srhs, sy, sb, true);  // b = b0 + L^{-T} L^{-1} r
+    linv_solve32<NT>(Lb, n, srhs, sy, sb, true);  // b = b0 + L^{-T} L^{-1} r
     const float c1 = (float)p.lambda * kLog2e;
     const float tl = 2.f * (float)p.lambda, cm = (float)(p.lambda * p.lambda);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-      const float4 xi = mf4[m0 + i];
-      const float bi = sb[i], ai = xi.w;
-      float X0 = 0.f, X1 = 0.f, X2 = 0.f;
-      for (int j = 0; j < n; ++j) {
-        if (j == i) continue;
-        const float4 xj = mf4[m0 + j];
-        const float dx = xi.x - xj.x, dy = xi.y - xj.y, dz = xi.z - xj.z;
-        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+    for (int i = tid; i < n; i += NT) {
+      // two samples j per packed instruction (j == i adds zero: its offset is zero)
+      const float bi = sb[i], ai = sx[3 * n4 + i];
+      const unsigned long long XI = f2pack(sx[i], sx[i]), YI = f2pack(sx[n4 + i], sx[n4 + i]);
+      const unsigned long long ZI = f2pack(sx[2 * n4 + i], sx[2 * n4 + i]);
+      const unsigned long long BI = f2pack(bi, bi), AI = f2pack(ai, ai), NC1 = f2pack(-c1, -c1);
+      const float cg = MATERN ? cm : tl;
+      const unsigned long long CG = f2pack(cg, cg);
+      unsigned long long S0 = 0ull, S1 = 0ull, S2 = 0ull;
+      auto pair = [&](int e, int j) { return *reinterpret_cast<const unsigned long long*>(sx + e * n4 + j); };
+#pragma unroll 2
+      for (int j = 0; j < n4; j += 2) {
+        const unsigned long long dx = f2sub(XI, pair(0, j)), dy = f2sub(YI, pair(1, j)), dz = f2sub(ZI, pair(2, j));
+        const float2 r2 = f2unpack(f2fma(dx, dx, f2fma(dy, dy, f2mul(dz, dz))));
         // grad_{x_i} A_ij = -cg w_ij (x_i - x_j): RBF cg w = 2 lambda K_ij, Matern lambda^2 e^{-lambda r_ij}
-        const float cw = MATERN ? cm * ex2(-c1 * sqrt_approx(r2)) : tl * ex2(-c1 * r2);
-        const float cf = cw * fmaf(bi, xj.w, sb[j] * ai);
-        X0 = fmaf(cf, dx, X0);
-        X1 = fmaf(cf, dy, X1);
-        X2 = fmaf(cf, dz, X2);
+        const float2 ev = f2unpack(f2mul(NC1, MATERN ? f2pack(sqrt_approx(r2.x), sqrt_approx(r2.y)) : f2pack(r2.x, r2.y)));
+        const unsigned long long cw = f2mul(CG, f2pack(ex2(ev.x), ex2(ev.y)));
+        const unsigned long long bj = *reinterpret_cast<const unsigned long long*>(sb + j);
+        const unsigned long long cf = f2mul(cw, f2fma(BI, pair(3, j), f2mul(bj, AI)));
+        S0 = f2fma(cf, dx, S0);
+        S1 = f2fma(cf, dy, S1);
+        S2 = f2fma(cf, dz, S2);
       }
-      const int gid = mgid[m0 + i];
-      atomicAdd(&d_x[(int64_t)gid * p.dim + 0], X0);
-      atomicAdd(&d_x[(int64_t)gid * p.dim + 1], X1);
-      if (p.dim == 3) atomicAdd(&d_x[(int64_t)gid * p.dim + 2], X2);
+      const float2 s0 = f2unpack(S0), s1 = f2unpack(S1), s2 = f2unpack(S2);
+      const float X0 = s0.x + s0.y, X1 = s1.x + s1.y, X2 = s2.x + s2.y;
+      const int gid = a.mgid[m0 + i];
+      atomicAdd(&a.d_x[(int64_t)gid * p.dim + 0], X0);
+      atomicAdd(&a.d_x[(int64_t)gid * p.dim + 1], X1);
+      if (p.dim == 3) atomicAdd(&a.d_x[(int64_t)gid * p.dim + 2], X2);
     }
     __syncthreads();
   }
@@ -532,11 +609,11 @@ ksdf_status run_backward(ksdf_ctx* c, const float* xq, int64_t Q, const int8_t* 
   double* abar = ptr<double>(c->ws[WS_BW]);
   cudaEvent_t e_b = prof_begin(c), e0 = prof_begin(c);
   KSDF_CUDA(c, cudaMemsetAsync(cnt, 0, sizeof(int64_t) * G, st));
+  KSDF_CUDA(c, cudaMemsetAsync(tot, 0, sizeof(int64_t) * 6, st));
   KSDF_CUDA(c, cudaMemsetAsync(abar, 0, sizeof(double) * (m.M + 1), st));
   if (Q <= kSmallQ) {
     launch(k_bw_group_small, 1, kSmallThreads, 0, st, winner, (int)Q, G, cnt, d_xq, p.dim, sorted, tiles, tot, stw);
   } else {
-    KSDF_CUDA(c, cudaMemsetAsync(tot, 0, sizeof(int64_t) * 4, st));
     launch(k_bw_count, ceil_div(Q, 256), 256, 0, st, winner, Q, G, rank, cnt, d_xq, p.dim, stw);
     KSDF_CUDA(c, scan_i64(cnt, off, G, nullptr, c->ws[WS_SCAN], st));
     launch(k_ntiles_w, ceil_div(G, 256), 256, 0, st, cnt, G, nt);
@@ -573,23 +650,40 @@ ksdf_status run_backward(ksdf_ctx* c, const float* xq, int64_t Q, const int8_t* 
   launch(kq, std::max(1, occ) * c->num_sms, kTQ, smem, st, a, xq, p);
   prof_end(c, e0, "backward.query");
   e0 = prof_begin(c);
-  // two size classes, so that the many small cells run with shared memory for their own size (more CTAs per SM
-  // to hide the factors' load latency); the larger cells beside them on an auxiliary stream
-  auto kc = matern ? k_bw_cell<true> : k_bw_cell<false>;
-  const int maxn = std::max(m.max_n, 1), nsplit = std::min(maxn, kBwCellSmallN);
-  const bool two = maxn > nsplit;
+  // two size classes, the larger cells beside the others on an auxiliary stream; their lists take the place of the tile
+  // counts and offsets, which are done with
+  const bool small = Q <= kSmallQ;
+  int32_t* list = reinterpret_cast<int32_t*>(nt);
+  int* ccnt = reinterpret_cast<int*>(tot + 4);
+  const int maxn = std::max(m.max_n, 1), bound = std::min(maxn, small ? kBwSmemN : kBwSplitN);
+  launch(k_bw_cells, ceil_div(G, 256), 256, 0, st, cnt, ptr<int32_t>(m.n), G, bound, list, ccnt);
+  const bool two = maxn > bound;
   if (two) KSDF_CUDA(c, fork_streams(c));
-  for (int part = 0; part < (two ? 2 : 1); ++part) {
-    const int nlo = part == 0 ? 0 : nsplit + 1, nhi = part == 0 ? nsplit : maxn;
-    const size_t smem2 = (sizeof(double) + sizeof(float)) * 3 * (size_t)nhi;
+  for (int part = two ? 1 : 0; part >= 0; --part) {
+    const bool sm = small && part == 0;
+    const size_t smem2 = bw_smem_bytes(part == 0 ? bound : maxn, sm);
+    const int threads = !small ? 64 : sm ? 128 : 256;
+    auto kc = !small ? (matern ? k_bw_cell<true, false, 64> : k_bw_cell<false, false, 64>)
+              : sm   ? (matern ? k_bw_cell<true, true, 128> : k_bw_cell<false, true, 128>)
+                     : (matern ? k_bw_cell<true, false, 256> : k_bw_cell<false, false, 256>);
     KSDF_CUDA(c, cudaFuncSetAttribute(kc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2));
     int occ2 = 0;
-    KSDF_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, kc, kBwCellThreads, smem2));
-    const unsigned grid2 = (unsigned)std::min<int64_t>(G, (int64_t)std::max(1, occ2) * c->num_sms);
-    launch(kc, std::max(1u, grid2), kBwCellThreads, smem2, part == 0 ? st : c->aux[0], cnt, G,
-           ptr<int64_t>(m.ts_off), ptr<int32_t>(m.n), ptr<int64_t>(m.chol_off), ptr<double>(m.chol64),
-           ptr<int64_t>(m.linv_off), ptr<float>(m.linv32), ptr<float4>(m.mf4), ptr<int32_t>(m.mgid), abar, p, d_x,
-           nlo, nhi);
+    KSDF_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ2, kc, threads, smem2));
+    BwCellArgs ca;
+    ca.list = list + part * G;
+    ca.count = ccnt + part;
+    ca.ts_off = ptr<int64_t>(m.ts_off);
+    ca.cell_n = ptr<int32_t>(m.n);
+    ca.chol_off = ptr<int64_t>(m.chol_off);
+    ca.chol64 = ptr<double>(m.chol64);
+    ca.linv_off = ptr<int64_t>(m.linv_off);
+    ca.linv32 = ptr<float>(m.linv32);
+    ca.mf4 = ptr<float4>(m.mf4);
+    ca.mgid = ptr<int32_t>(m.mgid);
+    ca.abar = abar;
+    ca.d_x = d_x;
+    const int64_t grid2 = std::min<int64_t>(std::min<int64_t>(G, Q), (int64_t)std::max(1, occ2) * c->num_sms);
+    launch(kc, (unsigned)grid2, threads, smem2, part == 0 ? st : c->aux[0], ca, p);
   }
   if (two) KSDF_CUDA(c, join_streams(c));
   KSDF_CUDA(c, cudaGetLastError());
