@@ -18,7 +18,7 @@ constexpr double kExpC1 = 0x1.62e42fefa39efp-17;
 constexpr double kExpC2 = 0x1.ebfbdff82c58fp-35;
 constexpr double kExpQ16PerNat = 0x1.71547652b82fep+16;
 
-__device__ double kExpT1[256] = {  // 2^(-j/256)
+static __device__ double kExpT1[256] = {  // 2^(-j/256)
     0x1.0000000000000p+0, 0x1.fe9d96b2a23d9p-1, 0x1.fd3c22b8f71f1p-1, 0x1.fbdba3692d514p-1,
     0x1.fa7c1819e90d8p-1, 0x1.f91d802243c89p-1, 0x1.f7bfdad9cbe14p-1, 0x1.f6632798844f8p-1,
     0x1.f50765b6e4540p-1, 0x1.f3ac948dd7274p-1, 0x1.f252b376bba97p-1, 0x1.f0f9c1cb6412ap-1,
@@ -84,7 +84,7 @@ __device__ double kExpT1[256] = {  // 2^(-j/256)
     0x1.059b0d3158574p-1, 0x1.04e5f72f654b1p-1, 0x1.04315e86e7f85p-1, 0x1.037d42e11bbccp-1,
     0x1.02c9a3e778061p-1, 0x1.02168143b0281p-1, 0x1.0163da9fb3335p-1, 0x1.00b1afa5abcbfp-1,
 };
-__device__ double kExpT2[256] = {  // 2^(-j/65536)
+static __device__ double kExpT2[256] = {  // 2^(-j/65536)
     0x1.0000000000000p+0, 0x1.fffe9d1c4b0f3p-1, 0x1.fffd3a398c1bbp-1, 0x1.fffbd757c324dp-1,
     0x1.fffa7476f029dp-1, 0x1.fff91197132a2p-1, 0x1.fff7aeb82c251p-1, 0x1.fff64bda3b19fp-1,
     0x1.fff4e8fd40081p-1, 0x1.fff386213aeedp-1, 0x1.fff223462bcd8p-1, 0x1.fff0c06c12a37p-1,
