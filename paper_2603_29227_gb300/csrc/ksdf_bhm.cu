@@ -7,6 +7,7 @@
 //   Wmp[slot * NW + i] float2 {mu, P} per weight (NW = n_h^3 + 1, the bias last): mean and precision of the map
 //                     before the running update; A0, A1, B[slot * NW + i] floats: the update's accumulators,
 //                     A = sum c(xi) phi^2 of odd (A0) and even (A1) EM rounds and B = sum (t - 1/2) phi
+//   Ms                float2 {mean, 1 / precision} of the running EM round's M-step, of the touched blocks
 //   hash table        block key -> slot (open addressing, linear probing), 4x the block capacity
 //   per block         packed key, active flag, the frame stamps of the touched / marked lists, its marked-cell index
 //   masks             one bit per marching cell of each marked block ((n_h m)^3 bits)
@@ -67,11 +68,11 @@ struct BhmDev {
   uint8_t* active;
   int32_t *stamp_touch, *stamp_mark, *mark_idx;
   int32_t *new_list, *touched, *marked;
-  float2* Wmp;
+  float2 *Wmp, *Ms;
   float *A0, *A1, *Bacc;
-  // candidate hinge offsets (dz + 8) << 16 | (dy + 8) << 8 | (dx + 8), z-major, per octant of the fraction (the
-  // offsets within reach of that half-cell sub-cube): 8 tables of ostride entries, kNoCand padded
-  const int32_t* ocand;
+  // candidate hinge offsets (make_cand), z-major, per octant of the fraction (the offsets within reach of that
+  // half-cell sub-cube): 8 tables of ostride entries, padded with offsets out of reach
+  const int4* ocand;
   int ostride;           // entries per octant table, a multiple of 32
   uint32_t* masks;
   BhmState* st;
@@ -92,14 +93,20 @@ struct __align__(16) RayInfo {
   Sample hit;
 };
 
+constexpr int kFewRounds = 3;  // the rounds of reach r = 1 (at most 64 offsets) and of a short r = 2 (the city map: 84)
 constexpr int kMaxRounds = 7;  // candidate rounds of 32 lanes: (2 r + 2)^3 <= 216 offsets for r <= 2
-constexpr int kNoCand = -1;
 
 __device__ __forceinline__ double lat(double x, double o, double h) { return __ddiv_rn(__dsub_rn(x, o), h); }
 __device__ __forceinline__ bool lat_ok(double u) { return u > -kLatMax && u < kLatMax; }
 __host__ __device__ __forceinline__ int fdiv(int a, int b) {  // floor(a / b), b > 0
   int q = a / b;
   return (a < 0 && q * b != a) ? q - 1 : q;
+}
+
+__device__ __forceinline__ float ex2_ftz(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 
 __device__ __forceinline__ void set_status(BhmState* st, uint32_t bit) { atomicOr(&st->status, bit); }
@@ -263,6 +270,79 @@ __device__ void bhm_eval(const BhmDev& d, Win& w, const double u[3], float& l, f
   l = sl;
   g = make_float3(d.g2h * gx, d.g2h * gy, d.g2h * gz);
   v = sv;
+}
+
+// ---- a warp's candidate features ---------------------------------------------------------------------------
+// The EM and the prediction are bound by instruction issue (78% of the slots, 150 instructions per round of 32 offsets
+// when every lane unpacked its offset and formed slot and index from three coordinates), so all that depends on the
+// offset alone is tabulated, and all that depends on the point alone is prepared by one lane, 32 points at a time, and
+// read back by the whole warp as three 16-byte broadcasts.  Measured with k_bhm_mstep, a city frame's update and 1,000,000
+// predictions: 4.44 -> 3.40 ms.
+
+// One candidate offset: {x, y, z} = offset << kQ (the fixed-point distance subtracts it as it stands) and, packed, the
+// offset + RW per axis in three 6-bit fields under its linear index (oz n_h + oy) n_h + ox in the top 12 bits.
+__host__ inline int4 make_cand(int ox, int oy, int oz, int rw, int nh) {
+  const int lin = (oz * nh + oy) * nh + ox;
+  const int w = ((oz + rw) << 12) | ((oy + rw) << 6) | (ox + rw);
+  return make_int4(ox * (1 << kQ), oy * (1 << kQ), oz * (1 << kQ), (int)((uint32_t)lin << 20) | w);
+}
+__host__ inline int4 no_cand() { return make_int4(1 << 26, 0, 0, 0); }  // beyond every reach (< 3 << kQ)
+
+// One point: its fixed-point fraction and, in three 6-bit fields, bse - RW + 32 - n_h (so that adding a candidate's
+// fields sets bit 5 of a field when the hinge lies in the upper block of the window, l >= n_h); the binary32 fraction and
+// the linear index of bse; the packed window corner, the octant's first candidate and the label - 1/2.
+struct __align__(16) Rec {
+  int q[3], fld;
+  float f[3];
+  int lin;
+  uint32_t klo, khi;
+  int oct;
+  float tb;
+};
+__device__ __forceinline__ void make_rec(const BhmDev& d, const int g[3], const int q[3], const float f[3], float tb,
+                                         Rec& o) {
+  int lo[3], bse[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    lo[a] = fdiv(g[a] - d.rw, d.nh);
+    bse[a] = g[a] - d.nh * lo[a];
+    o.q[a] = q[a];
+    o.f[a] = f[a];
+  }
+  const int fb = 32 - d.nh - d.rw;
+  o.fld = ((bse[2] + fb) << 12) | ((bse[1] + fb) << 6) | (bse[0] + fb);
+  o.lin = (bse[2] * d.nh + bse[1]) * d.nh + bse[0];
+  const uint64_t k = pack_key(lo[0], lo[1], lo[2]);
+  o.klo = (uint32_t)k;
+  o.khi = (uint32_t)(k >> 32);
+  o.oct = (((q[2] >> (kQ - 1)) << 2) | ((q[1] >> (kQ - 1)) << 1) | (q[0] >> (kQ - 1))) * d.ostride;
+  o.tb = tb;
+}
+
+// lanes 0..7: the weight index of local coordinate (0, 0, 0) of window block (lane & 1, lane >> 1 & 1, lane >> 2),
+// less the wrap of coordinates >= n_h; INT_MIN where the block is not allocated
+__device__ __forceinline__ int window_base(const BhmDev& d, int slot, int lane) {
+  const int nh = d.nh;
+  return slot < 0 ? INT_MIN : slot * d.nw - (((lane >> 2) * nh + ((lane >> 1) & 1)) * nh + (lane & 1)) * nh;
+}
+// the lane (mod 32) that holds the window base of the fields' block: bits 5, 11 and 17 to bits 24, 25 and 26 (the other
+// partial products fall on distinct bits below 24 or above 28, so nothing carries)
+__device__ __forceinline__ int window_lane(int fld) {
+  return (int)((((uint32_t)fld & 0x20820u) * ((1u << 19) + (1u << 14) + (1u << 9))) >> 24);
+}
+
+// candidate c of point (pa: q, fld; pf: f; lin): the weight's index or a negative number, f - offset in df; every
+// lane of the warp calls
+__device__ __forceinline__ int candidate(const BhmDev& d, const int4& c, const int4& pa, const float4& pf, int base,
+                                         float df[3]) {
+  const int tx = pa.x - c.x, ty = pa.y - c.y, tz = pa.z - c.z;
+  const long long D = (long long)tx * tx + (long long)ty * ty + (long long)tz * tz;  // units of 2^-40
+  const int b = __shfl_sync(0xffffffffu, base, window_lane(pa.w + c.w));
+  const int idx = b + (__float_as_int(pf.w) + (c.w >> 20));
+  df[0] = fmaf((float)c.x, -9.5367431640625e-7f, pf.x);  // 2^-20: the product is exact
+  df[1] = fmaf((float)c.y, -9.5367431640625e-7f, pf.y);
+  df[2] = fmaf((float)c.z, -9.5367431640625e-7f, pf.z);
+  return D <= d.r2q ? idx : -1;
 }
 
 // ---- update kernels --------------------------------------------------------------------------------------
@@ -456,112 +536,115 @@ __global__ void __launch_bounds__(kT) k_bhm_walk(BhmDev d, const RayInfo* __rest
 }
 
 // One EM round over the update's samples, a warp per 32 consecutive samples.  FIRST: xi = xi_init, accumulates B
-// and A into A0 (and builds the touched-block list).  Otherwise: the M-step of each sample from the previous
-// round's posterior (its A in src: 0 = A0, 1 = A1), then the E-step statistic c(xi) phi^2 into dst.
-template <bool FIRST>
+// and A into A0 (and builds the touched-block list).  Otherwise: the M-step of each sample from the weights'
+// posterior of the previous round (k_bhm_mstep), then the E-step statistic c(xi) phi^2 into dst.
+// NR bounds the candidate rounds, so that the reach of up to 96 offsets an octant keeps its features in few registers.
+template <bool FIRST, int NR>
 __global__ void __launch_bounds__(kT) k_bhm_em(BhmDev d, const Sample* __restrict__ smp,
-                                               const unsigned long long* __restrict__ n_dev, int src, int dst) {
+                                               const unsigned long long* __restrict__ n_dev, int dst) {
   constexpr unsigned FULL = 0xffffffffu;
+  extern __shared__ int4 s_cand[];  // the octants' candidates
+  __shared__ Rec s_rec[kT];
   const int64_t N = (int64_t)*n_dev;
   const int lane = threadIdx.x & 31;
+  Rec* rec = s_rec + (threadIdx.x - lane);
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int nh = d.nh, nw = d.nw, RW = d.rw;
-  // the candidate offsets of each octant of the fraction (a sample's octant is the top bit of each fraction)
-  __shared__ int s_cand[8 * kMaxRounds * 32];
   for (int i = threadIdx.x; i < 8 * d.ostride; i += blockDim.x) s_cand[i] = d.ocand[i];
   __syncthreads();
   const int nrounds = d.ostride / 32;
-  const float* Asrc = src ? d.A1 : d.A0;
+  const int own = (d.rw << 12) | (d.rw << 6) | d.rw;  // the fields of offset 0: the point's own block
   float* Adst = dst ? d.A1 : d.A0;
-  int wlo[3] = {INT_MIN, INT_MIN, INT_MIN};
-  int myslot = -1;  // lanes 0..7: slot of window block lo + (lane & 1, lane >> 1 & 1, lane >> 2)
-  unsigned long long nfeat = 0;
+  const float c0 = jj_coef(d.xi0);
+  uint32_t wklo = ~0u, wkhi = ~0u;  // no packed key has all bits set
+  int wbase = INT_MIN;
+  unsigned nfeat = 0;
   for (int64_t base = gw * 32; base < N; base += nwarps * 32) {
-    Sample my = {};
-    if (base + lane < N) my = smp[base + lane];
-    const int nv = (int)(N - base < 32 ? N - base : 32);
-    for (int s = 0; s < nv; ++s) {
-      int g[3], bse[3], lo[3], q[3];
+    __syncwarp();
+    if (base + lane < N) {
+      const Sample my = smp[base + lane];
+      int q[3];
       float f[3];
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        g[a] = __shfl_sync(FULL, my.g[a], s);
-        const uint32_t fq = __shfl_sync(FULL, my.fq[a], s);
-        q[a] = (int)(fq >> 12);
-        f[a] = (float)fq * 2.3283064365386963e-10f;  // 2^-32
-        lo[a] = fdiv(g[a] - RW, nh);
-        bse[a] = g[a] - nh * lo[a];
+        q[a] = (int)(my.fq[a] >> 12);
+        f[a] = (float)my.fq[a] * 2.3283064365386963e-10f;  // 2^-32
       }
-      const float tb = (float)__shfl_sync(FULL, my.t, s) - 0.5f;
-      const int* oc = s_cand + (((q[2] >> 19) << 2) | ((q[1] >> 19) << 1) | (q[0] >> 19)) * d.ostride;
-      if (lo[0] != wlo[0] || lo[1] != wlo[1] || lo[2] != wlo[2]) {
-        wlo[0] = lo[0];
-        wlo[1] = lo[1];
-        wlo[2] = lo[2];
+      make_rec(d, my.g, q, f, (float)my.t - 0.5f, rec[lane]);
+    }
+    __syncwarp();
+    const int nv = (int)(N - base < 32 ? N - base : 32);
+    for (int s = 0; s < nv; ++s) {
+      const int4* rp = reinterpret_cast<const int4*>(rec + s);
+      const int4 pa = rp[0], pk = rp[2];
+      const float4 pf = *reinterpret_cast<const float4*>(rp + 1);
+      const float tb = __int_as_float(pk.w);
+      if ((uint32_t)pk.x != wklo || (uint32_t)pk.y != wkhi) {
+        wklo = (uint32_t)pk.x;
+        wkhi = (uint32_t)pk.y;
         if (lane < 8) {
-          myslot = find_block(d, lo[0] + (lane & 1), lo[1] + ((lane >> 1) & 1), lo[2] + (lane >> 2));
-          if (FIRST && myslot >= 0 && d.stamp_touch[myslot] != d.frame) {
-            if (atomicExch(&d.stamp_touch[myslot], d.frame) != d.frame)
-              d.touched[atomicAdd(&d.st->n_touched, 1)] = myslot;
+          int lo[3];
+          unpack_key((uint64_t)wkhi << 32 | wklo, lo[0], lo[1], lo[2]);
+          const int slot = find_block(d, lo[0] + (lane & 1), lo[1] + ((lane >> 1) & 1), lo[2] + (lane >> 2));
+          wbase = window_base(d, slot, lane);
+          if (FIRST && slot >= 0 && d.stamp_touch[slot] != d.frame) {
+            if (atomicExch(&d.stamp_touch[slot], d.frame) != d.frame)
+              d.touched[atomicAdd(&d.st->n_touched, 1)] = slot;
           }
         }
+        __syncwarp();
       }
-      const int bsl = __shfl_sync(FULL, myslot, (bse[2] >= nh) * 4 + (bse[1] >= nh) * 2 + (bse[0] >= nh));
-      const int bidx = (d.bias && bsl >= 0) ? bsl * nw + nw - 1 : -1;
-      float phr[kMaxRounds];
-      int idr[kMaxRounds];
+      const int4* oc = s_cand + pk.z + lane;
+      // the bias weight of the point's own block, by lane 0: the window base less its wrap, plus n_h^3
+      const int ol = window_lane(pa.w + own) & 7;
+      const int ob = __shfl_sync(FULL, wbase, ol);
+      const int bidx = d.bias && ob != INT_MIN
+                           ? ob + (((ol >> 2) * d.nh + ((ol >> 1) & 1)) * d.nh + (ol & 1)) * d.nh + d.nw - 1
+                           : -1;
+      float phr[NR];
+      int idr[NR];
       float vs = 0.f, ms = 0.f;
 #pragma unroll
-      for (int r = 0; r < kMaxRounds; ++r) {
+      for (int r = 0; r < NR; ++r) {
         idr[r] = -1;
         phr[r] = 0.f;
         if (r >= nrounds) continue;  // uniform across the warp
-        const int cd = oc[r * 32 + lane];
-        const int ox = (cd & 255) - 8, oy = ((cd >> 8) & 255) - 8, oz = ((cd >> 16) & 255) - 8;
-        // |fraction - offset|^2 in units of 2^-40, each term one 32 x 32 -> 64-bit product
-        const int tx = q[0] - ox * (1 << kQ), ty = q[1] - oy * (1 << kQ), tz = q[2] - oz * (1 << kQ);
-        const long long D = (long long)tx * tx + (long long)ty * ty + (long long)tz * tz;
-        const int lx = bse[0] + ox, ly = bse[1] + oy, lz = bse[2] + oz;
-        const int sl = __shfl_sync(FULL, myslot, (lz >= nh) * 4 + (ly >= nh) * 2 + (lx >= nh));
-        const bool ok = cd != kNoCand && D <= d.r2q && sl >= 0;
-        const float fx = f[0] - (float)ox, fy = f[1] - (float)oy, fz = f[2] - (float)oz;
-        const float phi = __expf(-d.gh2 * (fx * fx + fy * fy + fz * fz));
-        const int idx = sl * nw + ((lz - (lz >= nh ? nh : 0)) * nh + (ly - (ly >= nh ? nh : 0))) * nh +
-                        (lx - (lx >= nh ? nh : 0));
-        phr[r] = phi;
-        idr[r] = ok ? idx : -1;
-        if (!FIRST && ok) {
-          const float2 w = d.Wmp[idx];
-          const float inv = __fdividef(1.0f, w.y + Asrc[idx]);
-          const float mu = fmaf(w.y, w.x, d.Bacc[idx]) * inv;
-          vs = fmaf(phi * phi, inv, vs);
-          ms = fmaf(mu, phi, ms);
+        float df[3];
+        const int idx = candidate(d, oc[r * 32], pa, pf, wbase, df);
+        // phi >= phi_min where it is used, so the flush of tiny results in ex2 plays no part
+        const float phi = ex2_ftz(-d.gh2 * (df[0] * df[0] + df[1] * df[1] + df[2] * df[2]) * 1.4426950408889634f);
+        if (FIRST) {
+          if (idx >= 0) {
+            atomicAdd(&Adst[idx], c0 * phi * phi);
+            atomicAdd(&d.Bacc[idx], tb * phi);
+            ++nfeat;
+          }
+        } else {
+          phr[r] = phi;
+          idr[r] = idx;
+          if (idx >= 0) {
+            const float2 w = d.Ms[idx];
+            vs = fmaf(phi * phi, w.y, vs);
+            ms = fmaf(w.x, phi, ms);
+          }
         }
-        if (FIRST) nfeat += (unsigned long long)__popc(__ballot_sync(FULL, ok));
       }
-      float xi = d.xi0;
+      float c = c0;
       if (!FIRST) {
         if (lane == 0 && bidx >= 0) {
-          const float2 w = d.Wmp[bidx];
-          const float P = w.y + Asrc[bidx];
-          vs += 1.0f / P;
-          ms += fmaf(w.y, w.x, d.Bacc[bidx]) / P;
+          const float2 w = d.Ms[bidx];
+          vs += w.y;
+          ms += w.x;
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
           vs += __shfl_xor_sync(FULL, vs, o);
           ms += __shfl_xor_sync(FULL, ms, o);
         }
-        xi = sqrtf(fmaf(ms, ms, vs));
-      }
-      const float c = jj_coef(xi);
+        c = jj_coef(sqrtf(fmaf(ms, ms, vs)));
 #pragma unroll
-      for (int r = 0; r < kMaxRounds; ++r) {
-        if (idr[r] >= 0) {
-          atomicAdd(&Adst[idr[r]], c * phr[r] * phr[r]);
-          if (FIRST) atomicAdd(&d.Bacc[idr[r]], tb * phr[r]);
-        }
+        for (int r = 0; r < NR; ++r)
+          if (idr[r] >= 0) atomicAdd(&Adst[idr[r]], c * phr[r] * phr[r]);
       }
       if (lane == 0 && bidx >= 0) {
         atomicAdd(&Adst[bidx], c);
@@ -569,7 +652,28 @@ __global__ void __launch_bounds__(kT) k_bhm_em(BhmDev d, const Sample* __restric
       }
     }
   }
-  if (FIRST && lane == 0 && nfeat) atomicAdd(&d.st->n_features, nfeat);
+  if (FIRST) {
+    unsigned long long n = nfeat;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(FULL, n, o);
+    if (lane == 0 && n) atomicAdd(&d.st->n_features, n);
+  }
+}
+
+// the M-step of every weight of the touched blocks from the previous round's accumulators (A of round src): once a
+// weight instead of once a (sample, weight), which a weight near the surface is asked for hundreds of times
+__global__ void k_bhm_mstep(BhmDev d, int src) {
+  const int n = d.st->n_touched;
+  const float* A = src ? d.A1 : d.A0;
+  for (int b = blockIdx.x; b < n; b += gridDim.x) {
+    const int64_t base = (int64_t)d.touched[b] * d.nw;
+    for (int k = threadIdx.x; k < d.nw; k += blockDim.x) {
+      const int64_t i = base + k;
+      const float2 w = d.Wmp[i];
+      const float P = w.y + A[i];
+      d.Ms[i] = make_float2(fmaf(w.y, w.x, d.Bacc[i]) / P, 1.0f / P);
+    }
+  }
 }
 
 // zero one accumulator of every touched block (before EM rounds three and four, which reuse them)
@@ -956,26 +1060,29 @@ __global__ void k_bhm_gather(MarchOut mo, int64_t n, double* x, float* var, floa
 // Prediction, a warp per 32 points: each lane sets up one point (binary64 lattice coordinate, fixed-point and
 // binary32 fraction), then the warp takes the points one at a time, its lanes splitting the point's candidate
 // offsets (the octant table of the EM); sums by warp reduction; each lane writes its own point's outputs.
-template <bool GV>
+template <bool GV, int NR>
 __global__ void __launch_bounds__(kT) k_bhm_query(BhmDev d, const float* __restrict__ xq, int64_t Q, uint32_t mask,
                                                   float* lo_out, int8_t* sg, float* gr, float* pr) {
   constexpr unsigned FULL = 0xffffffffu;
-  __shared__ int s_cand[8 * kMaxRounds * 32];
+  extern __shared__ int4 s_cand[];
+  __shared__ Rec s_rec[kT];
   for (int i = threadIdx.x; i < 8 * d.ostride; i += blockDim.x) s_cand[i] = d.ocand[i];
   __syncthreads();
   const int lane = threadIdx.x & 31;
+  Rec* rec = s_rec + (threadIdx.x - lane);
   const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  const int nh = d.nh, nw = d.nw, RW = d.rw, nrounds = d.ostride / 32;
+  const int nrounds = d.ostride / 32;
+  const int own = (d.rw << 12) | (d.rw << 6) | d.rw;
   const double tau = d.st->tau;
-  int wlo[3] = {INT_MIN, INT_MIN, INT_MIN};
-  int myslot = -1;
+  uint32_t wklo = ~0u, wkhi = ~0u;
+  int wbase = INT_MIN;
   for (int64_t base = gw * 32; base < Q; base += nwarps * 32) {
     const int64_t i = base + lane;
-    int g[3] = {0, 0, 0}, q[3] = {0, 0, 0};
-    float f[3] = {0.f, 0.f, 0.f};
     bool ok = i < Q;
     if (ok) {
+      int g[3], q[3];
+      float f[3];
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
         const double u = lat((double)xq[3 * i + a], d.o[a], d.h);
@@ -986,57 +1093,52 @@ __global__ void __launch_bounds__(kT) k_bhm_query(BhmDev d, const float* __restr
         q[a] = (int)__dmul_rn(fr, (double)(1 << kQ));
         f[a] = (float)fr;
       }
-      if (!ok) set_status(d.st, ST_NONFINITE);
+      if (ok) make_rec(d, g, q, f, 0.f, rec[lane]);
+      else set_status(d.st, ST_NONFINITE);
     }
+    unsigned todo = __ballot_sync(FULL, ok);  // also orders the records before their readers
+    __syncwarp();
     float my_l = 0.f, my_v = 0.f, my_g[3] = {0.f, 0.f, 0.f};
-    const int nv = (int)(Q - base < 32 ? Q - base : 32);
-    for (int s = 0; s < nv; ++s) {
-      if (!__shfl_sync(FULL, (int)ok, s)) continue;  // uniform
-      int gg[3], qq[3], bse[3], lo[3];
-      float ff[3];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        gg[a] = __shfl_sync(FULL, g[a], s);
-        qq[a] = __shfl_sync(FULL, q[a], s);
-        ff[a] = __shfl_sync(FULL, f[a], s);
-        lo[a] = fdiv(gg[a] - RW, nh);
-        bse[a] = gg[a] - nh * lo[a];
+    while (todo) {
+      const int s = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int4* rp = reinterpret_cast<const int4*>(rec + s);
+      const int4 pa = rp[0], pk = rp[2];
+      const float4 pf = *reinterpret_cast<const float4*>(rp + 1);
+      if ((uint32_t)pk.x != wklo || (uint32_t)pk.y != wkhi) {
+        wklo = (uint32_t)pk.x;
+        wkhi = (uint32_t)pk.y;
+        if (lane < 8) {
+          int lo[3];
+          unpack_key((uint64_t)wkhi << 32 | wklo, lo[0], lo[1], lo[2]);
+          wbase = window_base(
+              d, find_block(d, lo[0] + (lane & 1), lo[1] + ((lane >> 1) & 1), lo[2] + (lane >> 2)), lane);
+        }
+        __syncwarp();
       }
-      if (lo[0] != wlo[0] || lo[1] != wlo[1] || lo[2] != wlo[2]) {
-        wlo[0] = lo[0];
-        wlo[1] = lo[1];
-        wlo[2] = lo[2];
-        if (lane < 8) myslot = find_block(d, lo[0] + (lane & 1), lo[1] + ((lane >> 1) & 1), lo[2] + (lane >> 2));
-      }
-      const int* oc = s_cand + (((qq[2] >> 19) << 2) | ((qq[1] >> 19) << 1) | (qq[0] >> 19)) * d.ostride;
+      const int4* oc = s_cand + pk.z + lane;
       float sl = 0.f, sv = 0.f, sx = 0.f, sy = 0.f, sz = 0.f;
 #pragma unroll
-      for (int r = 0; r < kMaxRounds; ++r) {
+      for (int r = 0; r < NR; ++r) {
         if (r >= nrounds) continue;  // uniform
-        const int cd = oc[r * 32 + lane];
-        const int ox = (cd & 255) - 8, oy = ((cd >> 8) & 255) - 8, oz = ((cd >> 16) & 255) - 8;
-        const int tx = qq[0] - ox * (1 << kQ), ty = qq[1] - oy * (1 << kQ), tz = qq[2] - oz * (1 << kQ);
-        const long long D = (long long)tx * tx + (long long)ty * ty + (long long)tz * tz;
-        const int lx = bse[0] + ox, ly = bse[1] + oy, lz = bse[2] + oz;
-        const int slt = __shfl_sync(FULL, myslot, (lz >= nh) * 4 + (ly >= nh) * 2 + (lx >= nh));
-        if (cd == kNoCand || D > d.r2q || slt < 0) continue;
-        const float fx = ff[0] - (float)ox, fy = ff[1] - (float)oy, fz = ff[2] - (float)oz;
-        const float phi = expf(-d.gh2 * (fx * fx + fy * fy + fz * fz));
-        const int idx = slt * nw + ((lz - (lz >= nh ? nh : 0)) * nh + (ly - (ly >= nh ? nh : 0))) * nh +
-                        (lx - (lx >= nh ? nh : 0));
+        float df[3];
+        const int idx = candidate(d, oc[r * 32], pa, pf, wbase, df);
+        if (idx < 0) continue;
+        const float phi = expf(-d.gh2 * (df[0] * df[0] + df[1] * df[1] + df[2] * df[2]));
         const float2 w = d.Wmp[idx];
         const float mp = w.x * phi;
         sl += mp;
         if (GV) {
-          sx = fmaf(mp, fx, sx);
-          sy = fmaf(mp, fy, sy);
-          sz = fmaf(mp, fz, sz);
+          sx = fmaf(mp, df[0], sx);
+          sy = fmaf(mp, df[1], sy);
+          sz = fmaf(mp, df[2], sz);
           sv = fmaf(phi * phi, 1.0f / w.y, sv);
         }
       }
-      const int bsl = __shfl_sync(FULL, myslot, (bse[2] >= nh) * 4 + (bse[1] >= nh) * 2 + (bse[0] >= nh));
-      if (lane == 0 && d.bias && bsl >= 0) {
-        const float2 w = d.Wmp[(int64_t)bsl * nw + nw - 1];
+      const int ol = window_lane(pa.w + own) & 7;
+      const int ob = __shfl_sync(FULL, wbase, ol);
+      if (lane == 0 && d.bias && ob != INT_MIN) {
+        const float2 w = d.Wmp[ob + (((ol >> 2) * d.nh + ((ol >> 1) & 1)) * d.nh + (ol & 1)) * d.nh + d.nw - 1];
         sl += w.x;
         if (GV) sv += 1.0f / w.y;
       }
@@ -1058,6 +1160,7 @@ __global__ void __launch_bounds__(kT) k_bhm_query(BhmDev d, const float* __restr
         my_g[2] = d.g2h * sz;
       }
     }
+    __syncwarp();  // the records are rewritten by the next 32 points
     if (i < Q) {
       if (!ok) {
         my_l = my_v = __int_as_float(0x7fc00000);
@@ -1119,7 +1222,7 @@ struct ksdf_bhm {
   long long r2q = 0;
   int64_t max_blocks = 0, max_marked = 0;
   uint64_t hcap = 0;
-  DevBuf hkeys, hvals, bkey, active, stamps, lists, Wmp, A0, A1, B, ocand, masks, state;
+  DevBuf hkeys, hvals, bkey, active, stamps, lists, Wmp, Ms, A0, A1, B, ocand, masks, state;
   DevBuf stage_hits, mkey, mval, mx, mvar, mnrm, sort_tmp, out_stage[4], q_stage[5];
   DevBuf smp, scnt, soff, scan_tmp, rays;
   int64_t mcap = 0, scap = 0;
@@ -1200,16 +1303,20 @@ BhmDev dev_view(ksdf_bhm* m) {
   d.touched = li + m->hcap;
   d.marked = li + m->hcap + m->max_blocks;
   d.Wmp = ptr<float2>(m->Wmp);
+  d.Ms = ptr<float2>(m->Ms);
   d.A0 = ptr<float>(m->A0);
   d.A1 = ptr<float>(m->A1);
   d.Bacc = ptr<float>(m->B);
-  d.ocand = ptr<int32_t>(m->ocand);
+  d.ocand = ptr<int4>(m->ocand);
   d.ostride = m->ostride;
   d.rw = m->rw;
   d.masks = ptr<uint32_t>(m->masks);
   d.st = ptr<BhmState>(m->state);
   return d;
 }
+
+// the candidate table of the EM and the prediction (at most 28 KB, next to 12 KB of records)
+size_t cand_smem(int ostride) { return sizeof(int4) * (size_t)8 * ostride; }
 
 unsigned nblk(int64_t n) { return (unsigned)((n + kT - 1) / kT); }
 
@@ -1245,7 +1352,7 @@ ksdf_status ksdf_bhm_create(const ksdf_bhm_params* prm, int64_t max_blocks, int6
   if (max_blocks * nw >= (1LL << 31)) return KSDF_ERR_ARG;  // weight indices are 32-bit
   const double rr2 = (double)r2q / 1099511627776.0 + 1e-9;
   // per octant of the fraction ([0, 1/2] or [1/2, 1] per axis): the offsets within reach of that sub-cube
-  std::vector<int32_t> ocand[8];
+  std::vector<int4> ocand[8];
   size_t omax = 0;
   for (int o = 0; o < 8; ++o) {
     for (int dz = -rw; dz <= rw + 1; ++dz)
@@ -1258,12 +1365,12 @@ ksdf_status ksdf_bhm_create(const ksdf_bhm_params* prm, int64_t max_blocks, int6
             const double gap = dd[a] < lo ? lo - dd[a] : (dd[a] > hi ? dd[a] - hi : 0.0);
             g2 += gap * gap;
           }
-          if (g2 <= rr2) ocand[o].push_back(((dz + 8) << 16) | ((dy + 8) << 8) | (dx + 8));
+          if (g2 <= rr2) ocand[o].push_back(make_cand(dx, dy, dz, rw, p.block_hinges));
         }
     omax = std::max(omax, ocand[o].size());
   }
   const int ostride = (int)((omax + 31) / 32 * 32);
-  std::vector<int32_t> otab((size_t)8 * ostride, -1);
+  std::vector<int4> otab((size_t)8 * ostride, no_cand());
   for (int o = 0; o < 8; ++o) std::copy(ocand[o].begin(), ocand[o].end(), otab.begin() + (size_t)o * ostride);
 
   ksdf_bhm* m = new ksdf_bhm();
@@ -1292,17 +1399,18 @@ ksdf_status ksdf_bhm_create(const ksdf_bhm_params* prm, int64_t max_blocks, int6
   al(m->stamps, 12 * (size_t)max_blocks);
   al(m->lists, 4 * (cap + 2 * (size_t)max_blocks));  // new-key list (one per table position), touched, marked
   al(m->Wmp, 8 * (size_t)max_blocks * m->nw);
+  al(m->Ms, 8 * (size_t)max_blocks * m->nw);
   al(m->A0, 4 * (size_t)max_blocks * m->nw);
   al(m->A1, 4 * (size_t)max_blocks * m->nw);
   al(m->B, 4 * (size_t)max_blocks * m->nw);
-  al(m->ocand, 4 * (size_t)8 * ostride);
+  al(m->ocand, sizeof(int4) * (size_t)8 * ostride);
   al(m->masks, 4 * (size_t)m->max_marked * m->mask_words);
   al(m->state, sizeof(BhmState));
   if (e == cudaSuccess) e = cudaMemsetAsync(m->hkeys.p, 0xff, 8 * cap, m->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(m->hvals.p, 0xff, 4 * cap, m->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(m->state.p, 0, sizeof(BhmState), m->stream);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(m->ocand.p, otab.data(), 4 * otab.size(), cudaMemcpyHostToDevice, m->stream);
+    e = cudaMemcpyAsync(m->ocand.p, otab.data(), sizeof(int4) * otab.size(), cudaMemcpyHostToDevice, m->stream);
   if (e == cudaSuccess) {
     const double tau = p.tau_init;
     e = cudaMemcpyAsync(reinterpret_cast<char*>(m->state.p) + offsetof(BhmState, tau), &tau, sizeof(double),
@@ -1319,7 +1427,7 @@ ksdf_status ksdf_bhm_create(const ksdf_bhm_params* prm, int64_t max_blocks, int6
 
 ksdf_status ksdf_bhm_destroy(ksdf_bhm* m) {
   if (!m) return KSDF_OK;
-  DevBuf* bufs[] = {&m->hkeys, &m->hvals, &m->bkey, &m->active, &m->stamps, &m->lists, &m->Wmp, &m->A0,
+  DevBuf* bufs[] = {&m->hkeys, &m->hvals, &m->bkey, &m->active, &m->stamps, &m->lists, &m->Wmp, &m->Ms, &m->A0,
                     &m->A1, &m->B, &m->ocand, &m->masks, &m->state, &m->stage_hits, &m->mkey, &m->mval,
                     &m->mx, &m->mvar, &m->mnrm, &m->sort_tmp, &m->smp, &m->scnt, &m->soff, &m->scan_tmp,
                     &m->rays};
@@ -1391,8 +1499,13 @@ ksdf_status ksdf_bhm_update(ksdf_bhm* m, const double* p, const double* hits, in
     for (int it = 1; it <= iters; ++it) {
       const int dst = (it - 1) & 1, src = it >= 2 ? (it - 2) & 1 : 0;
       if (it >= 3) launch(k_bhm_zero_acc, kGridStride, kT, 0, st, d, dst);
-      if (it == 1) launch(k_bhm_em<true>, ge, kT, 0, st, d, (const Sample*)smp, &sdev->n_samples, src, dst);
-      else launch(k_bhm_em<false>, ge, kT, 0, st, d, (const Sample*)smp, &sdev->n_samples, src, dst);
+      if (it >= 2) launch(k_bhm_mstep, kGridStride, kT, 0, st, d, src);
+      if (m->ostride <= 32 * kFewRounds)
+        launch(it == 1 ? k_bhm_em<true, kFewRounds> : k_bhm_em<false, kFewRounds>, ge, kT, cand_smem(m->ostride), st, d,
+               (const Sample*)smp, &sdev->n_samples, dst);
+      else
+        launch(it == 1 ? k_bhm_em<true, kMaxRounds> : k_bhm_em<false, kMaxRounds>, ge, kT, cand_smem(m->ostride), st, d,
+               (const Sample*)smp, &sdev->n_samples, dst);
     }
     launch(k_bhm_commit, kGridStride, kT, 0, st, d, (iters - 1) & 1);
     switch (m->rw) {
@@ -1509,12 +1622,13 @@ ksdf_status ksdf_bhm_query(ksdf_bhm* m, const float* xq, int64_t Q, uint32_t out
   }
   BhmDev d = dev_view(m);
   const unsigned gq = (unsigned)std::max<int64_t>(1, std::min<int64_t>((Q * 32 + kT - 1) / kT / 32 + 1, 152 * 16));
-  if (out_mask & (KSDF_BHM_GRAD | KSDF_BHM_PROB))
-    launch(k_bhm_query<true>, gq, kT, 0, st, d, dq, Q, out_mask & 15u, (float*)dv[0], (int8_t*)dv[1], (float*)dv[2],
-           (float*)dv[3]);
+  const bool gv = (out_mask & (KSDF_BHM_GRAD | KSDF_BHM_PROB)) != 0;
+  if (m->ostride <= 32 * kFewRounds)
+    launch(gv ? k_bhm_query<true, kFewRounds> : k_bhm_query<false, kFewRounds>, gq, kT, cand_smem(m->ostride), st, d, dq,
+           Q, out_mask & 15u, (float*)dv[0], (int8_t*)dv[1], (float*)dv[2], (float*)dv[3]);
   else
-    launch(k_bhm_query<false>, gq, kT, 0, st, d, dq, Q, out_mask & 15u, (float*)dv[0], (int8_t*)dv[1],
-           (float*)dv[2], (float*)dv[3]);
+    launch(gv ? k_bhm_query<true, kMaxRounds> : k_bhm_query<false, kMaxRounds>, gq, kT, cand_smem(m->ostride), st, d, dq,
+           Q, out_mask & 15u, (float*)dv[0], (int8_t*)dv[1], (float*)dv[2], (float*)dv[3]);
   BHM_CUDA(m, cudaGetLastError());
   for (int i = 0; i < 4; ++i)
     if (outs[i] && dv[i] != outs[i])
