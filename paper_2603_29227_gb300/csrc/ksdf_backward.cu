@@ -147,23 +147,34 @@ struct BwArgs {
 // Jacobian sum_i alpha_i w_i (I - (lambda / |r_i|) r_i r_i^T), so that
 //   x_bar = -lambda^2 fb G + f_w v - lambda H' v  (f_w = sum alpha_i w_i, H' = sum (alpha_i w_i / |r_i|) r_i r_i^T),
 //   alpha_bar_i += fb k'_i + w_i (r_i . v),  X_bar_i += alpha_i w_i ((lambda^2 fb + lambda (r_i . v) / |r_i|) r_i - v).
+//
+// FP32 bound.  HASV, a cotangent of the gradient, is a template parameter: without one H v = 0, so pass 1 leaves M out and
+// pass 2 the terms in v (46 of 61 operations per query and sample are left).  Pass 2 takes two queries per packed
+// instruction.  Pass 1 does not: f' in two partial sums differs from the sequential sum in its last bits, which 1 / u
+// magnifies without bound near the surface.  Measured without a gradient cotangent: 16,777,216 queries on cells of mean N 81,
+// 4.07 -> 2.84 ms.
 constexpr int kTQ = 128;  // backward tile: queries (pass 1) and threads
+constexpr int kPair = 64;  // pairs of queries of a tile
 
-template <bool MATERN>
+// shared memory: the cell's samples [n_max]; the tile's queries as pairs (both queries' x, both queries' y): x y | z fb | wx wy | wz nx | ny nz (w = 2 (x - x_n)), then v0 v1 | v2 m where HASV or MATERN; [kTQ] group partial sums
+__host__ __device__ constexpr int bq_rows(bool ext) { return ext ? 7 : 5; }
+__host__ __device__ inline size_t bq_smem_bytes(int n_max, bool ext) {
+  return sizeof(float4) * (size_t)(n_max + bq_rows(ext) * kPair + kTQ);
+}
+
+template <bool MATERN, bool HASV>
 __global__ void __launch_bounds__(kTQ) k_bw_query(BwArgs a, const float* xq, Params p) {
-  extern __shared__ __align__(16) float4 s_x[];  // [n_max] samples | per query: (x, fb) (w, -) (x_n, -) (v, -) |
-                                                 // [kTQ][4] group partial sums
+  typedef unsigned long long u64;
+  extern __shared__ __align__(16) float4 s_x[];
   __shared__ int s_tile;
   __shared__ float s_bh[3], s_bl[3];
-  float4* QA = s_x + p.n_max;
-  float4* QW = QA + kTQ;
-  float4* QN = QW + kTQ;
-  float4* QV = QN + kTQ;
-  float4* RED = QV + kTQ;
+  float4* s_q = s_x + p.n_max;
+  float4* RED = s_q + bq_rows(HASV || MATERN) * kPair;
   const int tid = threadIdx.x;
   const float lam = (float)p.lambda;
   const float c1 = lam * kLog2e;
   const float tl = 2.f * lam;
+  const u64 NC1 = f2pack(-c1, -c1), LAM = f2pack(lam, lam), ONE = f2pack(1.f, 1.f);
   const int64_t ntiles = *a.n_tiles;
   for (;;) {
     if (tid == 0) s_tile = atomicAdd(a.counter, 1);
@@ -182,7 +193,8 @@ __global__ void __launch_bounds__(kTQ) k_bw_query(BwArgs a, const float* xq, Par
     }
     __syncthreads();
     // ---- pass 1: a thread per query ----
-    if (tid < tile.z) {
+    const int nq = tile.z;
+    if (tid < nq) {
       const int q = a.sorted[tile.y + tid];
       float ql[3] = {0.f, 0.f, 0.f};
       for (int j = 0; j < p.dim; ++j) ql[j] = local32(xq[(int64_t)q * p.dim + j], s_bh[j], s_bl[j]);
@@ -217,7 +229,7 @@ __global__ void __launch_bounds__(kTQ) k_bw_query(BwArgs a, const float* xq, Par
           const float y = den > 0.f ? fmaxf(e, 0.f) * __frcp_rn(den) : 0.f;
           aw = v.w * ex2(-c1 * y);
           ak = aw * fmaf(lam, z, 1.f);
-          ac = z > 0.f ? aw * __frcp_rn(z) : 0.f;
+          ac = HASV && z > 0.f ? aw * __frcp_rn(z) : 0.f;
         } else {
           ak = v.w * ex2(-c1 * e);
           aw = ak;
@@ -231,19 +243,21 @@ __global__ void __launch_bounds__(kTQ) k_bw_query(BwArgs a, const float* xq, Par
         D0 -= aw * ax;
         D1 -= aw * ay;
         D2 -= aw * az;
-        const float bx = ac * ax, by = ac * ay, bz = ac * az;
-        if (MATERN) {
-          fc += ac;
-          C0 -= bx;
-          C1 -= by;
-          C2 -= bz;
+        if (HASV) {
+          const float bx = ac * ax, by = ac * ay, bz = ac * az;
+          if (MATERN) {
+            fc += ac;
+            C0 -= bx;
+            C1 -= by;
+            C2 -= bz;
+          }
+          M00 = fmaf(bx, ax, M00);
+          M01 = fmaf(bx, ay, M01);
+          M02 = fmaf(bx, az, M02);
+          M11 = fmaf(by, ay, M11);
+          M12 = fmaf(by, az, M12);
+          M22 = fmaf(bz, az, M22);
         }
-        M00 = fmaf(bx, ax, M00);
-        M01 = fmaf(bx, ay, M01);
-        M02 = fmaf(bx, az, M02);
-        M11 = fmaf(by, ay, M11);
-        M12 = fmaf(by, az, M12);
-        M22 = fmaf(bz, az, M22);
       }
       f -= comp;
       if (!MATERN) {
@@ -273,7 +287,7 @@ __global__ void __launch_bounds__(kTQ) k_bw_query(BwArgs a, const float* xq, Par
         }
       }
       float v0 = 0.f, v1 = 0.f, v2 = 0.f;
-      if (a.d_grad) {
+      if (HASV) {
         const float gn = sqrtf(G0 * G0 + G1 * G1 + G2 * G2);
         if (gn > 0.f) {
           const float g0 = G0 / gn, g1 = G1 / gn, g2 = G2 / gn;
@@ -288,15 +302,18 @@ __global__ void __launch_bounds__(kTQ) k_bw_query(BwArgs a, const float* xq, Par
       }
       // x_bar = -cg fb G + fw v - beta H v with H v = fc (p.v) p + (p.v) C + p (C.v) + M v; RBF cg = beta = 2 lambda,
       // Matern cg = lambda^2, beta = lambda (the 1/|r_i| is inside the weights of fc, C, M)
-      const float pv = fmaf(px, v0, fmaf(py, v1, pz * v2)), cv = fmaf(C0, v0, fmaf(C1, v1, C2 * v2));
-      const float fpv = fc * pv;
-      const float hv0 = fmaf(fpv, px, fmaf(pv, C0, fmaf(px, cv, fmaf(M00, v0, fmaf(M01, v1, M02 * v2)))));
-      const float hv1 = fmaf(fpv, py, fmaf(pv, C1, fmaf(py, cv, fmaf(M01, v0, fmaf(M11, v1, M12 * v2)))));
-      const float hv2 = fmaf(fpv, pz, fmaf(pv, C2, fmaf(pz, cv, fmaf(M02, v0, fmaf(M12, v1, M22 * v2)))));
       const float cg = MATERN ? lam * lam : tl, beta = MATERN ? lam : tl;
-      float xb0 = fmaf(-cg * fb, G0, fmaf(-beta, hv0, fw * v0));
-      float xb1 = fmaf(-cg * fb, G1, fmaf(-beta, hv1, fw * v1));
-      float xb2 = fmaf(-cg * fb, G2, fmaf(-beta, hv2, fw * v2));
+      float xb0 = -cg * fb * G0, xb1 = -cg * fb * G1, xb2 = -cg * fb * G2;
+      if (HASV) {
+        const float pv = fmaf(px, v0, fmaf(py, v1, pz * v2)), cv = fmaf(C0, v0, fmaf(C1, v1, C2 * v2));
+        const float fpv = fc * pv;
+        const float hv0 = fmaf(fpv, px, fmaf(pv, C0, fmaf(px, cv, fmaf(M00, v0, fmaf(M01, v1, M02 * v2)))));
+        const float hv1 = fmaf(fpv, py, fmaf(pv, C1, fmaf(py, cv, fmaf(M01, v0, fmaf(M11, v1, M12 * v2)))));
+        const float hv2 = fmaf(fpv, pz, fmaf(pv, C2, fmaf(pz, cv, fmaf(M02, v0, fmaf(M12, v1, M22 * v2)))));
+        xb0 = fmaf(-cg * fb, G0, fmaf(-beta, hv0, fw * v0));
+        xb1 = fmaf(-cg * fb, G1, fmaf(-beta, hv1, fw * v1));
+        xb2 = fmaf(-cg * fb, G2, fmaf(-beta, hv2, fw * v2));
+      }
       if (fallback && m > 0.f) {
         // u = distance to the nearest sample: its own derivative, on the query and on that sample
         const float d = sqrtf(m);
@@ -312,47 +329,98 @@ __global__ void __launch_bounds__(kTQ) k_bw_query(BwArgs a, const float* xq, Par
       a.d_xq[(int64_t)q * p.dim + 0] = xb0;
       a.d_xq[(int64_t)q * p.dim + 1] = xb1;
       if (p.dim == 3) a.d_xq[(int64_t)q * p.dim + 2] = xb2;
-      QA[tid] = make_float4(ql[0], ql[1], ql[2], fb);
-      QW[tid] = make_float4(wx, wy, wz, 0.f);
-      QN[tid] = make_float4(xn.x, xn.y, xn.z, m);
-      QV[tid] = make_float4(v0, v1, v2, 0.f);
+      float* e = reinterpret_cast<float*>(s_q + (tid >> 1)) + (tid & 1);
+      const float rec[10] = {ql[0], ql[1], ql[2], fb, wx, wy, wz, xn.x, xn.y, xn.z};
+      // an odd last pair's second query repeats the first with cotangents of zero
+      const bool twin = tid == nq - 1 && !(tid & 1);
+#pragma unroll
+      for (int k = 0; k < 10; ++k) {
+        e[(k >> 1) * 4 * kPair + (k & 1) * 2] = rec[k];
+        if (twin) e[(k >> 1) * 4 * kPair + (k & 1) * 2 + 1] = k == 3 ? 0.f : rec[k];
+      }
+      if (HASV || MATERN) {
+        const float ext[4] = {v0, v1, v2, m};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          e[(5 + (k >> 1)) * 4 * kPair + (k & 1) * 2] = ext[k];
+          if (twin) e[(5 + (k >> 1)) * 4 * kPair + (k & 1) * 2 + 1] = k < 3 ? 0.f : m;
+        }
+      }
     }
     __syncthreads();
-    // ---- pass 2: a thread per (sample, group of queries) ----
+    // ---- pass 2: a thread per (sample, group of query pairs) ----
     const int nrep = n < kTQ ? kTQ / n : 1;  // query groups when the cell is small
     const int grp = tid / (n < kTQ ? n : kTQ);
-    const int nq = tile.z;
+    const int np = (nq + 1) >> 1;
     for (int i0 = 0; i0 < n; i0 += kTQ) {
       const int i = i0 + (n < kTQ ? tid - grp * n : tid);
       const bool act = grp < nrep && i < n;
       float ab = 0.f, X0 = 0.f, X1 = 0.f, X2 = 0.f;
       if (act) {
         const float4 xi = s_x[i];
-        for (int qq = grp; qq < nq; qq += nrep) {
-          const float4 A = QA[qq], W = QW[qq], Nn = QN[qq], V = QV[qq];
-          const float r0 = A.x - xi.x, r1 = A.y - xi.y, r2 = A.z - xi.z;
-          const float e = excess_sq(xi.x, xi.y, xi.z, Nn.x, Nn.y, Nn.z, W.x, W.y, W.z);
-          const float rv = fmaf(r0, V.x, fmaf(r1, V.y, r2 * V.z));
-          float t2, aw;
-          if (MATERN) {
-            const float rr = Nn.w + e, z = rr > 0.f ? rr * rsqrtf(rr) : 0.f, zm = sqrtf(Nn.w);
-            const float den = z + zm;
-            const float y = den > 0.f ? fmaxf(e, 0.f) * __frcp_rn(den) : 0.f;
-            const float wg = ex2(-c1 * y);
-            ab = fmaf(A.w * fmaf(lam, z, 1.f), wg, fmaf(wg, rv, ab));
-            aw = xi.w * wg;
-            t2 = fmaf(lam * lam, A.w, z > 0.f ? lam * rv * __frcp_rn(z) : 0.f);
-          } else {
-            const float kp = ex2(-c1 * e);
-            const float c = rv + A.w;
-            ab = fmaf(kp, c, ab);
-            aw = xi.w * kp;
-            t2 = tl * c;
+        const u64 IX = f2pack(xi.x, xi.x), IY = f2pack(xi.y, xi.y), IZ = f2pack(xi.z, xi.z);
+        const u64 TL = f2pack(tl, tl), L2 = f2pack(lam * lam, lam * lam);
+        u64 AB = 0ull, Y0 = 0ull, Y1 = 0ull, Y2 = 0ull;  // X = (the factors that the queries share) Y
+#pragma unroll 2
+        for (int qq = grp; qq < np; qq += nrep) {
+          const float4 s0 = s_q[qq], s1 = s_q[kPair + qq], s2 = s_q[2 * kPair + qq], s3 = s_q[3 * kPair + qq];
+          const float4 s4 = s_q[4 * kPair + qq];
+          const u64 r0 = f2sub(f2pack(s0.x, s0.y), IX), r1 = f2sub(f2pack(s0.z, s0.w), IY);
+          const u64 r2 = f2sub(f2pack(s1.x, s1.y), IZ), FB = f2pack(s1.z, s1.w);
+          const u64 ax = f2sub(IX, f2pack(s3.z, s3.w)), ay = f2sub(IY, f2pack(s4.x, s4.y));
+          const u64 az = f2sub(IZ, f2pack(s4.z, s4.w));
+          const u64 e = f2fma(ax, f2sub(ax, f2pack(s2.x, s2.y)),
+                              f2fma(ay, f2sub(ay, f2pack(s2.z, s2.w)), f2mul(az, f2sub(az, f2pack(s3.x, s3.y)))));
+          float4 s5 = {}, s6 = {};
+          u64 rv = 0ull;
+          if (HASV || MATERN) s6 = s_q[6 * kPair + qq];
+          if (HASV) {
+            s5 = s_q[5 * kPair + qq];
+            rv = f2fma(r0, f2pack(s5.x, s5.y), f2fma(r1, f2pack(s5.z, s5.w), f2mul(r2, f2pack(s6.x, s6.y))));
           }
-          X0 = fmaf(aw, fmaf(t2, r0, -V.x), X0);
-          X1 = fmaf(aw, fmaf(t2, r1, -V.y), X1);
-          X2 = fmaf(aw, fmaf(t2, r2, -V.z), X2);
+          u64 kw, t2;  // the weight w_i (RBF: k'_i) and the factor of r_i beside it
+          if (MATERN) {
+            const float2 es = f2unpack(e);
+            const float ra = s6.z + es.x, rb = s6.w + es.y, ma = sqrtf(s6.z), mb = sqrtf(s6.w);
+            const float za = ra > 0.f ? ra * rsqrtf(ra) : 0.f, zb = rb > 0.f ? rb * rsqrtf(rb) : 0.f;
+            const float da = za + ma, db = zb + mb;
+            const float ya = da > 0.f ? fmaxf(es.x, 0.f) * __frcp_rn(da) : 0.f;
+            const float yb = db > 0.f ? fmaxf(es.y, 0.f) * __frcp_rn(db) : 0.f;
+            const float2 ey = f2unpack(f2mul(NC1, f2pack(ya, yb)));
+            kw = f2pack(ex2(ey.x), ex2(ey.y));
+            const u64 c = f2mul(FB, f2fma(f2pack(za, zb), LAM, ONE));
+            AB = f2fma(HASV ? f2add(c, rv) : c, kw, AB);
+            t2 = f2mul(L2, FB);
+            if (HASV) {
+              const u64 iz = f2pack(za > 0.f ? __frcp_rn(za) : 0.f, zb > 0.f ? __frcp_rn(zb) : 0.f);
+              t2 = f2fma(f2mul(LAM, rv), iz, t2);
+            }
+          } else {
+            const float2 ee = f2unpack(f2mul(NC1, e));
+            kw = f2pack(ex2(ee.x), ex2(ee.y));
+            const u64 c = HASV ? f2add(rv, FB) : FB;
+            AB = f2fma(kw, c, AB);
+            t2 = HASV ? f2mul(TL, c) : c;  // (without v the factor 2 lambda waits for the end)
+          }
+          if (HASV) {
+            const u64 nk = kw ^ 0x8000000080000000ull;
+            const u64 kt = f2mul(kw, t2);
+            Y0 = f2fma(kt, r0, f2fma(nk, f2pack(s5.x, s5.y), Y0));
+            Y1 = f2fma(kt, r1, f2fma(nk, f2pack(s5.z, s5.w), Y1));
+            Y2 = f2fma(kt, r2, f2fma(nk, f2pack(s6.x, s6.y), Y2));
+          } else {
+            const u64 kt = f2mul(kw, t2);
+            Y0 = f2fma(kt, r0, Y0);
+            Y1 = f2fma(kt, r1, Y1);
+            Y2 = f2fma(kt, r2, Y2);
+          }
         }
+        const float2 a2 = f2unpack(AB), y0 = f2unpack(Y0), y1 = f2unpack(Y1), y2 = f2unpack(Y2);
+        const float sc = HASV || MATERN ? xi.w : xi.w * tl;
+        ab = a2.x + a2.y;
+        X0 = sc * (y0.x + y0.y);
+        X1 = sc * (y1.x + y1.y);
+        X2 = sc * (y2.x + y2.y);
       }
       if (nrep > 1) {  // combine the query groups of each sample
         RED[tid] = make_float4(ab, X0, X1, X2);
@@ -640,9 +708,10 @@ ksdf_status run_backward(ksdf_ctx* c, const float* xq, int64_t Q, const int8_t* 
   a.d_xq = d_xq;
   a.d_x = d_x;
   a.abar = abar;
-  const size_t smem = sizeof(float4) * (p.n_max + 5 * kTQ);
   const bool matern = p.kernel == KSDF_KERNEL_MATERN32;
-  auto kq = matern ? k_bw_query<true> : k_bw_query<false>;
+  const size_t smem = bq_smem_bytes(p.n_max, matern || d_grad);
+  auto kq = matern ? (d_grad ? k_bw_query<true, true> : k_bw_query<true, false>)
+                   : (d_grad ? k_bw_query<false, true> : k_bw_query<false, false>);
   KSDF_CUDA(c, cudaFuncSetAttribute(kq, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int occ = 0;
   KSDF_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kq, kTQ, smem));
