@@ -1263,6 +1263,40 @@ __global__ void __launch_bounds__(kLbThreads) k_linv_big(LinvArgs a) {
 
 }  // namespace
 
+// what the query needs to tell from a distance that a cell cannot win (k_phaseA): a warp per cell
+__global__ void __launch_bounds__(256) k_bounds(const int32_t* n32, const int64_t* ts_off, const float4* mf4, int64_t G,
+                                                float4* bnd) {
+  const int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (g >= G) return;
+  const int n = n32[g];
+  const float4* v = mf4 + ts_off[g];
+  float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY}, P = 0.f;
+  for (int i = lane; i < n; i += 32) {
+    const float4 s = v[i];
+    lo[0] = fminf(lo[0], s.x);
+    lo[1] = fminf(lo[1], s.y);
+    lo[2] = fminf(lo[2], s.z);
+    hi[0] = fmaxf(hi[0], s.x);
+    hi[1] = fmaxf(hi[1], s.y);
+    hi[2] = fmaxf(hi[2], s.z);
+    P += s.w > 0.f || s.w != s.w ? s.w : 0.f;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      lo[j] = fminf(lo[j], __shfl_xor_sync(0xffffffffu, lo[j], o));
+      hi[j] = fmaxf(hi[j], __shfl_xor_sync(0xffffffffu, hi[j], o));
+    }
+    P += __shfl_xor_sync(0xffffffffu, P, o);
+  }
+  if (lane == 0) {
+    bnd[2 * g] = make_float4(lo[0], lo[1], lo[2], P == P ? logf(P) : INFINITY);
+    bnd[2 * g + 1] = make_float4(hi[0], hi[1], hi[2], 0.f);
+  }
+}
+
 static int bits_for(uint64_t v) {
   int b = 0;
   while (b < 64 && (v >> b) != 0) ++b;
@@ -1718,6 +1752,9 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
     ca.status = ptr<int32_t>(m.status);
     launch(k_copy_fit, (unsigned)std::min<int64_t>(G, 8 * c->num_sms), 256, 0, st, ca);
   }
+  KSDF_CUDA(c, ensure(m.bnd, sizeof(float4) * 2 * (G + 1)));
+  launch(k_bounds, ceil_div(G, 8), 256, 0, st, ptr<int32_t>(m.n), ptr<int64_t>(m.ts_off), ptr<float4>(m.mf4), G,
+         ptr<float4>(m.bnd));
   launch(k_sched_after, ceil_div(G, 256), 256, 0, st, (const int32_t*)touched, G, ptr<int32_t>(m.qc0),
          ptr<int32_t>(m.qc2), ptr<int32_t>(m.refit));
   // bricks over the cell bounding box for the candidate search (OK cells only; statuses are final here)

@@ -177,6 +177,7 @@ struct Model {
   DevBuf cell_order;                            // cells sorted by descending N (fit work order)
   // per member (CSR by ts_off)
   DevBuf mf4;      // float4 (x, y, z, alpha) cell-local, FP32
+  DevBuf bnd;      // float4 x 2 per cell: the box of mf4's positions (lo, hi), log of the sum of the positive alpha in lo.w
   DevBuf md4;      // D4 (x, y, z, alpha) cell-local, FP64
   DevBuf mvar;     // float sigma^2
   DevBuf mnrm;     // float4 normal
