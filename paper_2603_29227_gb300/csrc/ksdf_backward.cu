@@ -39,19 +39,17 @@ __device__ __forceinline__ float sqrt_approx(float x) {
 
 __global__ void k_bw_count(const int32_t* winner, int64_t Q, int64_t G, int32_t* rank, int64_t* cnt, float* d_xq,
                            int dim, uint32_t* st) {
-  int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= Q) return;
-  int w = winner[q];
+  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int w = q < Q ? winner[q] : -1;
   if (w >= G) {
     atomicOr(st, ST_CAPACITY);
     w = -1;
   }
-  if (w < 0) {
+  const int r = warp_rank(cnt, w < 0 ? -1 : w);
+  if (q >= Q) return;
+  rank[q] = w < 0 ? -1 : r;
+  if (w < 0)
     for (int j = 0; j < dim; ++j) d_xq[q * dim + j] = 0.f;
-    rank[q] = -1;
-    return;
-  }
-  rank[q] = (int32_t)atomicAdd((unsigned long long*)&cnt[w], 1ull);
 }
 
 __global__ void k_bw_scatter(const int32_t* winner, const int32_t* rank, int64_t Q, int64_t G, const int64_t* off,
@@ -683,9 +681,9 @@ ksdf_status run_backward(ksdf_ctx* c, const float* xq, int64_t Q, const int8_t* 
     launch(k_bw_group_small, 1, kSmallThreads, 0, st, winner, (int)Q, G, cnt, d_xq, p.dim, sorted, tiles, tot, stw);
   } else {
     launch(k_bw_count, ceil_div(Q, 256), 256, 0, st, winner, Q, G, rank, cnt, d_xq, p.dim, stw);
-    KSDF_CUDA(c, scan_i64(cnt, off, G, nullptr, c->ws[WS_SCAN], st));
     launch(k_ntiles_w, ceil_div(G, 256), 256, 0, st, cnt, G, nt);
-    KSDF_CUDA(c, scan_i64(nt, toff, G, &tot[0], c->ws[WS_SCAN], st));
+    const ScanJob jobs[2] = {{cnt, off, G, nullptr, nullptr, nullptr}, {nt, toff, G, &tot[0], nullptr, nullptr}};
+    KSDF_CUDA(c, scan_i64(jobs, 2, c->ws[WS_SCAN], st));
     launch(k_bw_scatter, ceil_div(Q, 256), 256, 0, st, winner, rank, Q, G, off, sorted);
     launch(k_bw_tiles, ceil_div(G, 256), 256, 0, st, cnt, off, toff, G, tiles);
   }

@@ -1463,10 +1463,11 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
     }
   }
   launch(k_sizes, ceil_div(G, 256), 256, 0, st, n64, G, tri64, lb64, tc64, ptr<int32_t>(m.n));
-  KSDF_CUDA(c, scan_i64(n64, ptr<int64_t>(m.ts_off), G, dtot, c->ws[WS_SCAN], st));
-  KSDF_CUDA(c, scan_i64(tri64, ptr<int64_t>(m.chol_off), G, dtot + 1, c->ws[WS_SCAN], st));
-  KSDF_CUDA(c, scan_i64(lb64, ptr<int64_t>(m.linv_off), G, dtot + 2, c->ws[WS_SCAN], st));
-  KSDF_CUDA(c, scan_i64(tc64, ptr<int64_t>(m.ltc_off), G, dtot + 3, c->ws[WS_SCAN], st));
+  const ScanJob jobs[4] = {{n64, ptr<int64_t>(m.ts_off), G, dtot, nullptr, nullptr},
+                           {tri64, ptr<int64_t>(m.chol_off), G, dtot + 1, nullptr, nullptr},
+                           {lb64, ptr<int64_t>(m.linv_off), G, dtot + 2, nullptr, nullptr},
+                           {tc64, ptr<int64_t>(m.ltc_off), G, dtot + 3, nullptr, nullptr}};
+  KSDF_CUDA(c, scan_i64(jobs, 4, c->ws[WS_SCAN], st));
   int64_t tots[4];
   int hmax[2];
   KSDF_CUDA(c, cudaMemcpyAsync(tots, dtot, sizeof(tots), cudaMemcpyDeviceToHost, st));

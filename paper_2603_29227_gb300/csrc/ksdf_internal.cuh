@@ -108,6 +108,16 @@ __device__ __forceinline__ float excess_sq(float vx, float vy, float vz, float n
   return fmaf(ax, ax - wx, fmaf(ay, ay - wy, az * (az - wz)));
 }
 
+// the lane's rank in group g (negative: none) of cnt, which counts it; a warp's lanes of one group take one atomic (the
+// queries of a batch's neighbours mostly have the same winner).  Every lane of the warp calls.
+__device__ __forceinline__ int warp_rank(int64_t* cnt, int g) {
+  const unsigned grp = __match_any_sync(0xffffffffu, g);
+  const int lane = threadIdx.x & 31, leader = __ffs(grp) - 1;
+  int base = 0;
+  if (lane == leader && g >= 0) base = (int)atomicAdd((unsigned long long*)&cnt[g], (unsigned long long)__popc(grp));
+  return __shfl_sync(0xffffffffu, base, leader) + __popc(grp & ((1u << lane) - 1u));
+}
+
 // hash of a packed key (splitmix64 finaliser)
 __host__ __device__ inline uint64_t mix64(uint64_t z) {
   z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
@@ -299,6 +309,18 @@ cudaError_t join_streams(ksdf_ctx* c);
 // n_dev (optional, a device count) only the first min(n, *n_dev) elements are scanned.
 cudaError_t scan_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* total, DevBuf& tmp, cudaStream_t st,
                      const int64_t* n_dev = nullptr);
+// the same of up to kMaxScanJobs arrays at once (their lengths alike: the launches are sized for the longest)
+constexpr int kMaxScanJobs = 4;
+struct ScanJob {
+  const int64_t* in;
+  int64_t* out;
+  int64_t n;
+  int64_t* total;
+  const int64_t* n_dev;
+  int64_t* sums;  // set by scan_i64
+};
+inline int64_t scan_sums_len(int64_t n) { return n / 2048 + 2; }  // block sums of one array in `tmp`
+cudaError_t scan_i64(const ScanJob* jobs, int nj, DevBuf& tmp, cudaStream_t st);
 // stable LSD radix sort by the low `bits` bits of 64-bit keys, with 32-bit values.  Result in keys/vals.
 cudaError_t radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int bits, DevBuf& tmp, cudaStream_t st);
 
@@ -332,7 +354,7 @@ enum WsRole {
   WS_D = 5,
   WS_E = 6,
   WS_F = 7,
-  WS_QKEY = 8,   // per query
+  WS_QSLOT = 8,  // per query
   WS_QBIN = 9,
   WS_QRANK = 10,
   WS_QSORT = 11,

@@ -3,6 +3,8 @@
 // enough.
 #include "ksdf_internal.cuh"
 
+#include <algorithm>
+
 namespace ksdf {
 
 namespace {
@@ -43,9 +45,18 @@ __device__ __forceinline__ int64_t scan_len(int64_t n, const int64_t* n_dev) {
   return n_dev ? (*n_dev < n ? *n_dev : n) : n;
 }
 
-__global__ void k_scan_reduce(const int64_t* in, int64_t n, const int64_t* n_dev, int64_t* sums) {
+// Several arrays are scanned by the same launches, one per blockIdx.y (the query's groupings scan two and four at a time:
+// at most sizes each launch is latency only).
+struct ScanJobs {
+  ScanJob j[kMaxScanJobs];
+};
+
+__global__ void k_scan_reduce(ScanJobs jobs) {
   __shared__ int64_t sw[kScanThreads / 32];
-  n = scan_len(n, n_dev);
+  const ScanJob& job = jobs.j[blockIdx.y];
+  const int64_t* in = job.in;
+  const int64_t n = scan_len(job.n, job.n_dev);
+  if ((int64_t)blockIdx.x * kScanTile >= n) return;  // the whole block is past the end (uniform)
   int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
   int64_t s = 0;
 #pragma unroll
@@ -53,11 +64,14 @@ __global__ void k_scan_reduce(const int64_t* in, int64_t n, const int64_t* n_dev
     if (base + i < n) s += in[base + i];
   int64_t tot;
   block_exscan(s, sw, &tot);
-  if (threadIdx.x == 0) sums[blockIdx.x] = tot;
+  if (threadIdx.x == 0) job.sums[blockIdx.x] = tot;
 }
 
-__global__ void k_scan_sums(int64_t* sums, int64_t nb, int64_t* total) {
+__global__ void k_scan_sums(ScanJobs jobs) {
   __shared__ int64_t sw[kScanThreads / 32];
+  const ScanJob& job = jobs.j[blockIdx.y];
+  int64_t* sums = job.sums;
+  const int64_t nb = (scan_len(job.n, job.n_dev) + kScanTile - 1) / kScanTile;
   int64_t carry = 0;
   for (int64_t c0 = 0; c0 < nb; c0 += kScanThreads) {
     int64_t i = c0 + threadIdx.x;
@@ -67,12 +81,15 @@ __global__ void k_scan_sums(int64_t* sums, int64_t nb, int64_t* total) {
     if (i < nb) sums[i] = carry + ex;
     carry += tot;
   }
-  if (threadIdx.x == 0 && total) *total = carry;
+  if (threadIdx.x == 0 && job.total) *job.total = carry;
 }
 
-__global__ void k_scan_apply(const int64_t* in, int64_t* out, int64_t n, const int64_t* n_dev, const int64_t* sums) {
+__global__ void k_scan_apply(ScanJobs jobs) {
   __shared__ int64_t sw[kScanThreads / 32];
-  n = scan_len(n, n_dev);
+  const ScanJob& job = jobs.j[blockIdx.y];
+  const int64_t* in = job.in;
+  int64_t* out = job.out;
+  const int64_t n = scan_len(job.n, job.n_dev);
   if ((int64_t)blockIdx.x * kScanTile >= n) return;  // the whole block is past the end (uniform)
   int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
   int64_t v[kScanItems];
@@ -83,7 +100,7 @@ __global__ void k_scan_apply(const int64_t* in, int64_t* out, int64_t n, const i
     s += v[i];
   }
   int64_t tot;
-  int64_t ex = block_exscan(s, sw, &tot) + sums[blockIdx.x];
+  int64_t ex = block_exscan(s, sw, &tot) + job.sums[blockIdx.x];
 #pragma unroll
   for (int i = 0; i < kScanItems; ++i) {
     if (base + i < n) out[base + i] = ex;
@@ -98,11 +115,13 @@ __global__ void k_scan_apply(const int64_t* in, int64_t* out, int64_t n, const i
 constexpr int kScanSingleThreads = 1024;
 constexpr int kScanSingleItems = 64;
 
-__global__ void __launch_bounds__(kScanSingleThreads) k_scan_single(const int64_t* in, int64_t* out, int64_t n,
-                                                                     const int64_t* n_dev, int64_t* total) {
+__global__ void __launch_bounds__(kScanSingleThreads) k_scan_single(ScanJobs jobs) {
   constexpr unsigned FULL = 0xffffffffu;
   __shared__ int64_t sw[kScanSingleThreads / 32];
-  n = scan_len(n, n_dev);
+  const ScanJob& job = jobs.j[blockIdx.y];
+  const int64_t* in = job.in;
+  int64_t* out = job.out;
+  const int64_t n = scan_len(job.n, job.n_dev);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t per = 32 * ((n + kScanSingleThreads - 1) / kScanSingleThreads);  // elements of a warp
   const int64_t b = warp * per, e = b + per < n ? b + per : n;
@@ -121,7 +140,7 @@ __global__ void __launch_bounds__(kScanSingleThreads) k_scan_single(const int64_
       if (lane >= o) w += y;
     }
     sw[lane] = w;  // inclusive prefix over the warps
-    if (lane == 31 && total) *total = w;
+    if (lane == 31 && job.total) *job.total = w;
   }
   __syncthreads();
   int64_t run = warp ? sw[warp - 1] : 0;
@@ -212,24 +231,51 @@ __global__ void k_rs_scatter(const uint64_t* keys, const uint32_t* vals, uint64_
 
 }  // namespace
 
+// the launches of a scan whose jobs have their sums
+static void scan_launch(const ScanJobs& js, int nj, int64_t n, cudaStream_t st) {
+  const unsigned y = (unsigned)nj;
+  if (n <= (int64_t)kScanSingleThreads * kScanSingleItems) {
+    launch(k_scan_single, dim3(1, y), kScanSingleThreads, 0, st, js);
+    return;
+  }
+  const unsigned nb = (unsigned)((n + kScanTile - 1) / kScanTile);
+  launch(k_scan_reduce, dim3(nb, y), kScanThreads, 0, st, js);
+  launch(k_scan_sums, dim3(1, y), kScanThreads, 0, st, js);
+  launch(k_scan_apply, dim3(nb, y), kScanThreads, 0, st, js);
+}
+
+cudaError_t scan_i64(const ScanJob* jobs, int nj, DevBuf& tmp, cudaStream_t st) {
+  ScanJobs js{};
+  int64_t n = 0, sums = 0;
+  int k = 0;
+  for (int i = 0; i < nj; ++i) {
+    if (jobs[i].n > 0) {
+      js.j[k++] = jobs[i];
+      n = std::max(n, jobs[i].n);
+      sums += scan_sums_len(jobs[i].n);
+    } else if (jobs[i].total) {
+      cudaError_t e = cudaMemsetAsync(jobs[i].total, 0, sizeof(int64_t), st);
+      if (e != cudaSuccess) return e;
+    }
+  }
+  if (k == 0) return cudaSuccess;
+  if (n > (int64_t)kScanSingleThreads * kScanSingleItems) {
+    cudaError_t e = ensure(tmp, sizeof(int64_t) * (size_t)sums);
+    if (e != cudaSuccess) return e;
+    int64_t* p = ptr<int64_t>(tmp);
+    for (int i = 0; i < k; ++i) {
+      js.j[i].sums = p;
+      p += scan_sums_len(js.j[i].n);
+    }
+  }
+  scan_launch(js, k, n, st);
+  return cudaGetLastError();
+}
+
 cudaError_t scan_i64(const int64_t* in, int64_t* out, int64_t n, int64_t* total, DevBuf& tmp, cudaStream_t st,
                      const int64_t* n_dev) {
-  if (n <= 0) {
-    if (total) return cudaMemsetAsync(total, 0, sizeof(int64_t), st);
-    return cudaSuccess;
-  }
-  if (n <= (int64_t)kScanSingleThreads * kScanSingleItems) {
-    launch(k_scan_single, 1, kScanSingleThreads, 0, st, in, out, n, n_dev, total);
-    return cudaGetLastError();
-  }
-  int64_t nb = (n + kScanTile - 1) / kScanTile;
-  cudaError_t e = ensure(tmp, sizeof(int64_t) * (size_t)(nb + 1));
-  if (e != cudaSuccess) return e;
-  int64_t* sums = ptr<int64_t>(tmp);
-  launch(k_scan_reduce, (unsigned)nb, kScanThreads, 0, st, in, n, n_dev, sums);
-  launch(k_scan_sums, 1, kScanThreads, 0, st, sums, nb, total);
-  launch(k_scan_apply, (unsigned)nb, kScanThreads, 0, st, in, out, n, n_dev, sums);
-  return cudaGetLastError();
+  const ScanJob job{in, out, n, total, n_dev, nullptr};
+  return scan_i64(&job, 1, tmp, st);
 }
 
 cudaError_t radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int bits, DevBuf& tmp, cudaStream_t st) {
@@ -254,13 +300,9 @@ cudaError_t radix_sort_u64(uint64_t* keys, uint32_t* vals, int64_t n, int bits, 
   for (int p = 0; p < passes; ++p) {
     int shift = 8 * p;
     launch(k_rs_hist, nblocks, kRsThreads, 0, st, ki, n, shift, hist, nblocks);
-    if (nh <= (int64_t)kScanSingleThreads * kScanSingleItems) {
-      launch(k_scan_single, 1, kScanSingleThreads, 0, st, hist, hist, nh, (const int64_t*)nullptr, (int64_t*)nullptr);
-    } else {
-      launch(k_scan_reduce, (unsigned)nb_scan, kScanThreads, 0, st, hist, nh, (const int64_t*)nullptr, sums);
-      launch(k_scan_sums, 1, kScanThreads, 0, st, sums, nb_scan, (int64_t*)nullptr);
-      launch(k_scan_apply, (unsigned)nb_scan, kScanThreads, 0, st, hist, hist, nh, (const int64_t*)nullptr, sums);
-    }
+    ScanJobs js{};
+    js.j[0] = ScanJob{hist, hist, nh, nullptr, nullptr, sums};
+    scan_launch(js, 1, nh, st);
     launch(k_rs_scatter, nblocks, kRsThreads, 0, st, ki, vi, ko, vo, n, shift, hist, nblocks);
     uint64_t* tk = ki; ki = ko; ko = tk;
     uint32_t* tv = vi; vi = vo; vo = tv;
