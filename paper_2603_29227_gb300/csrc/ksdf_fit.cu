@@ -135,81 +135,152 @@ __device__ void smem_bitonic(int* a, int n) {
   }
 }
 
-// training set of one cell per CTA: collection-box members, ascending global id, rank-selected cap.  128
-// threads: the neighbour cells' scans spread over four warps, and a cell's candidates (tens to a few
-// hundred) sort with few idle threads at the bitonic network's barriers
+// training set of one cell per CTA: collection-box members, ascending global id, rank-selected cap.  Bound by
+// instruction issue: 32 neighbour cells are looked up at once, a lane each, and the threads take their samples as one
+// run (a cell holds a few dozen, so a warp per neighbour left lanes idle and waited for each lookup in turn); up to
+// kRankN ids are ranked by counting the smaller ones, four compares per load and no barriers, above that the bitonic
+// network's n log^2 n is less than n^2.  Measured, 81,700 cells of mean N 80: 1.67 -> 0.54 ms (865 cells of mean N 473 0.23 -> 0.27).
 constexpr int kAssembleThreads = 128;
-__global__ void __launch_bounds__(kAssembleThreads) k_assemble(const uint64_t* cell_key, int64_t G, const int64_t* own_off,
-                                                  const uint32_t* own_id, const double* x, Params p, int R,
-                                                  const uint64_t* hk, const int32_t* hv, uint64_t hcap,
-                                                  int32_t* mpad, int64_t* n_out, int32_t* status, int* max_n,
-                                                  uint32_t* st) {
-  __shared__ int ids[kMaxPre];
-  __shared__ int cnt;
+constexpr int kRankN = 256;
+// Almost no cell has more than kSmallPre box members, and the ids of kMaxPre would leave room for six CTAs per SM: those
+// few cells go to a list that the second launch (REST) takes.
+constexpr int kSmallPre = 1024;
+template <bool REST>
+__global__ void __launch_bounds__(kAssembleThreads, REST ? 4 : 12)
+    k_assemble(const uint64_t* cell_key, int64_t G, const int64_t* own_off, const uint32_t* own_id, const double* x, Params p,
+               int R, const uint64_t* hk, const int32_t* hv, uint64_t hcap, int32_t* mpad, int64_t* n_out, int32_t* status,
+               int* max_n, uint32_t* st, int32_t* list, int* list_n) {
+  constexpr int CAP = REST ? kMaxPre : kSmallPre, kU = 2;
+  __shared__ __align__(16) int ids[CAP];
+  __shared__ int s_sorted[kRankN];
+  __shared__ int cnt, s_start[33];
+  __shared__ int64_t s_first[32];
   __shared__ long long s_lo[3], s_hi[3];
-  const int64_t g = blockIdx.x;
-  if (g >= G) return;
-  int c[3];
-  unpack_key(cell_key[g], c[0], c[1], c[2]);
-  // the box [lo, hi) in binary64 (computed once), compared through order-preserving integer keys
-  if (threadIdx.x == 0) {
-    cnt = 0;
-    for (int j = 0; j < 3; ++j) {
-      s_lo[j] = f64_order_key(__dsub_rn(cell_base(p.o[j], c[j], p.h), p.mu));
-      s_hi[j] = f64_order_key(__dadd_rn(cell_base(p.o[j], c[j] + 1, p.h), p.mu));
-    }
-  }
-  __syncthreads();
-  const long long lo[3] = {s_lo[0], s_lo[1], s_lo[2]}, hi[3] = {s_hi[0], s_hi[1], s_hi[2]};
-  // neighbour cells are spread over the warps (their hash lookups and member scans overlap)
-  const int side = 2 * R + 1, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  const int nnb = p.dim == 3 ? side * side * side : side * side;
-  for (int v = threadIdx.x >> 5; v < nnb; v += nwarps) {
-    const int dx = v % side - R, dy = (v / side) % side - R, dz = p.dim == 3 ? v / (side * side) - R : 0;
-    int64_t nb[3] = {(int64_t)c[0] + dx, (int64_t)c[1] + dy, (int64_t)c[2] + dz};
-    bool inr = true;
-    for (int j = 0; j < 3; ++j) inr &= nb[j] >= -kBias && nb[j] < kBias;
-    if (!inr) continue;
-    const int h = hash_find(hk, hv, hcap, pack_key(nb[0], nb[1], nb[2]));
-    if (h < 0) continue;
-    for (int64_t t = own_off[h] + lane; t < own_off[h + 1]; t += 32) {
-      const uint32_t id = own_id[t];
-      const double* xi = x + (int64_t)id * p.dim;
-      bool in = true;
-      for (int j = 0; j < p.dim; ++j) {
-        const long long k = f64_order_key(xi[j]);
-        in &= (k >= lo[j]) && (k < hi[j]);
-      }
-      if (in) {
-        const int pos = atomicAdd(&cnt, 1);
-        if (pos < kMaxPre) ids[pos] = (int)id;
-      }
-    }
-  }
-  __syncthreads();
-  int n = cnt;
-  if (n > kMaxPre) {
+  const int64_t cells = REST ? (int64_t)*list_n : G;
+  for (int64_t el = blockIdx.x; el < cells; el += gridDim.x) {
+    const int64_t g = REST ? (int64_t)list[el] : el;
+    __syncthreads();
+    int c[3];
+    unpack_key(cell_key[g], c[0], c[1], c[2]);
+    // the box [lo, hi) in binary64 (computed once), compared through order-preserving integer keys
     if (threadIdx.x == 0) {
-      atomicOr(st, ST_CAPACITY);
-      n_out[g] = 0;
-      status[g] = KSDF_CELL_EMPTY;
+      cnt = 0;
+      for (int j = 0; j < 3; ++j) {
+        s_lo[j] = f64_order_key(__dsub_rn(cell_base(p.o[j], c[j], p.h), p.mu));
+        s_hi[j] = f64_order_key(__dadd_rn(cell_base(p.o[j], c[j] + 1, p.h), p.mu));
+      }
     }
-    return;
-  }
-  int np2 = 1;
-  while (np2 < n) np2 <<= 1;
-  for (int i = n + threadIdx.x; i < np2; i += blockDim.x) ids[i] = INT32_MAX;
-  __syncthreads();
-  smem_bitonic(ids, np2);
-  int keep = n > p.n_max ? p.n_max : n;
-  for (int j = threadIdx.x; j < keep; j += blockDim.x) {
-    int src = n > p.n_max ? (int)(((int64_t)j * n) / p.n_max) : j;
-    mpad[g * p.n_max + j] = ids[src];
-  }
-  if (threadIdx.x == 0) {
-    n_out[g] = keep;
-    status[g] = keep > 0 ? KSDF_CELL_OK : KSDF_CELL_EMPTY;
-    atomicMax(max_n, keep);
+    __syncthreads();
+    const int side = 2 * R + 1, lane = threadIdx.x & 31;
+    const int nnb = p.dim == 3 ? side * side * side : side * side;
+    for (int v0 = 0; v0 < nnb; v0 += 32) {
+      if (threadIdx.x < 32) {
+        const int v = v0 + lane;
+        int len = 0;
+        int64_t first = 0;
+        if (v < nnb) {
+          const int dx = v % side - R, dy = (v / side) % side - R, dz = p.dim == 3 ? v / (side * side) - R : 0;
+          const int64_t nb[3] = {(int64_t)c[0] + dx, (int64_t)c[1] + dy, (int64_t)c[2] + dz};
+          bool inr = true;
+          for (int j = 0; j < 3; ++j) inr &= nb[j] >= -kBias && nb[j] < kBias;
+          const int h = inr ? hash_find(hk, hv, hcap, pack_key(nb[0], nb[1], nb[2])) : -1;
+          if (h >= 0) {
+            first = own_off[h];
+            len = (int)(own_off[h + 1] - first);
+          }
+        }
+        int e = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(0xffffffffu, e, o);
+          if (lane >= o) e += y;
+        }
+        s_start[lane + 1] = e;
+        s_first[lane] = first - (e - len);
+        if (lane == 0) s_start[0] = 0;
+      }
+      __syncthreads();
+      const int total = s_start[32];
+      for (int t0 = threadIdx.x - lane; t0 < total; t0 += kU * kAssembleThreads) {  // whole warps, kU loads in flight
+        uint32_t id[kU];
+        bool in[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          const int t = t0 + u * kAssembleThreads + lane;
+          in[u] = t < total;
+          int seg = 0;  // the last neighbour whose run starts at or before t
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1)
+            if (s_start[seg + o] <= t) seg += o;
+          id[u] = in[u] ? own_id[s_first[seg] + t] : 0u;
+        }
+        double v[kU][3];
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+#pragma unroll
+          for (int j = 0; j < 3; ++j) v[u][j] = j < p.dim ? x[(int64_t)id[u] * p.dim + j] : 0.0;
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            const long long k = f64_order_key(v[u][j]);
+            if (j < p.dim) in[u] &= (k >= s_lo[j]) && (k < s_hi[j]);
+          }
+          const unsigned bal = __ballot_sync(0xffffffffu, in[u]);
+          if (bal == 0) continue;
+          int pos = 0;
+          if (lane == 0) pos = atomicAdd(&cnt, __popc(bal));
+          pos = __shfl_sync(0xffffffffu, pos, 0) + __popc(bal & ((1u << lane) - 1u));
+          if (in[u] && pos < CAP) ids[pos] = (int)id[u];
+        }
+      }
+      __syncthreads();
+    }
+    int n = cnt;
+    if (n > CAP) {
+      if (!REST) {
+        if (threadIdx.x == 0) list[atomicAdd(list_n, 1)] = (int32_t)g;
+      } else if (threadIdx.x == 0) {
+        atomicOr(st, ST_CAPACITY);
+        n_out[g] = 0;
+        status[g] = KSDF_CELL_EMPTY;
+      }
+      continue;
+    }
+    const int* sorted = ids;
+    if (n <= kRankN) {
+      const int n4 = (n + 3) & ~3;
+      if (threadIdx.x < n4 - n) ids[n + threadIdx.x] = INT32_MAX;
+      __syncthreads();
+      for (int i = threadIdx.x; i < n; i += kAssembleThreads) {
+        const int own = ids[i];
+        int r = 0;
+#pragma unroll 4
+        for (int j = 0; j < n4; j += 4) {
+          const int4 o = *reinterpret_cast<const int4*>(ids + j);
+          r += (o.x < own) + (o.y < own) + (o.z < own) + (o.w < own);
+        }
+        s_sorted[r] = own;
+      }
+      __syncthreads();
+      sorted = s_sorted;
+    } else {
+      int np2 = 1;
+      while (np2 < n) np2 <<= 1;
+      for (int i = n + threadIdx.x; i < np2; i += blockDim.x) ids[i] = INT32_MAX;
+      __syncthreads();
+      smem_bitonic(ids, np2);
+    }
+    int keep = n > p.n_max ? p.n_max : n;
+    for (int j = threadIdx.x; j < keep; j += blockDim.x) {
+      int src = n > p.n_max ? (int)(((int64_t)j * n) / p.n_max) : j;
+      mpad[g * p.n_max + j] = sorted[src];
+    }
+    if (threadIdx.x == 0) {
+      n_out[g] = keep;
+      status[g] = keep > 0 ? KSDF_CELL_OK : KSDF_CELL_EMPTY;
+      atomicMax(max_n, keep);
+    }
   }
 }
 
@@ -1369,7 +1440,7 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
   // 1. bin
   KSDF_CUDA(c, ensure(c->ws[WS_A], sizeof(uint64_t) * S));
   KSDF_CUDA(c, ensure(c->ws[WS_B], sizeof(uint32_t) * S));
-  KSDF_CUDA(c, ensure(c->ws[WS_C], sizeof(int) * 8));
+  KSDF_CUDA(c, ensure(c->ws[WS_C], sizeof(int) * 12));
   uint64_t* keys = ptr<uint64_t>(c->ws[WS_A]);
   uint32_t* vals = ptr<uint32_t>(c->ws[WS_B]);
   int* bbox = ptr<int>(c->ws[WS_C]);
@@ -1432,9 +1503,12 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
   int64_t* lb64 = tri64 + (G + 1);
   int64_t* tc64 = lb64 + (G + 1);
   int* dmax = bbox + 6;
-  KSDF_CUDA(c, cudaMemsetAsync(dmax, 0, sizeof(int) * 2, st));
-  launch(k_assemble, (unsigned)G, kAssembleThreads, 0, st, ptr<uint64_t>(m.key), G, own_off, vals, x, p, R, ptr<uint64_t>(m.hkeys),
-         ptr<int32_t>(m.hvals), cap, ptr<int32_t>(m.mpad), n64, ptr<int32_t>(m.status), dmax, stw);
+  KSDF_CUDA(c, cudaMemsetAsync(dmax, 0, sizeof(int) * 3, st));
+  KSDF_CUDA(c, ensure(m.cell_order, sizeof(uint32_t) * (G + 1)));  // (holds the list of cells with many members until it is written)
+  for (int r = 0; r < 2; ++r)
+    launch(r ? k_assemble<true> : k_assemble<false>, (unsigned)(r ? std::min<int64_t>(G, 4 * c->num_sms) : G), kAssembleThreads, 0, st,
+           ptr<uint64_t>(m.key), G, own_off, vals, x, p, R, ptr<uint64_t>(m.hkeys), ptr<int32_t>(m.hvals), cap,
+           ptr<int32_t>(m.mpad), n64, ptr<int32_t>(m.status), dmax, stw, ptr<int32_t>(m.cell_order), dmax + 2);
   // refit scheduling: carried counters; with a budget, the changed cells beyond it keep their previous training
   // set (and, below, their previous fit)
   KSDF_CUDA(c, ensure(m.qc0, sizeof(int32_t) * (G + 1)));
