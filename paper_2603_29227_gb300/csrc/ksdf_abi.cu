@@ -244,7 +244,7 @@ static void release_model(Model& m) {
   DevBuf* bufs[] = {&m.key,   &m.status, &m.n,      &m.ts_off, &m.chol_off, &m.linv_off, &m.hkeys,
                     &m.hvals, &m.cell_order, &m.mf4, &m.bnd, &m.md4,    &m.mvar,     &m.mnrm,     &m.mgid,
                     &m.mpad,  &m.chol64, &m.linv32,  &m.x,      &m.ltc_off,  &m.ltc,      &m.var_all,
-                    &m.nrm_all, &m.bk_off, &m.bk_cells, &m.qc0,     &m.qc2,      &m.refit};
+                    &m.nrm_all, &m.bk_off, &m.bk_cells, &m.bk_keys, &m.qc0,     &m.qc2,      &m.refit};
   for (DevBuf* b : bufs) release(*b);
 }
 

@@ -1401,30 +1401,33 @@ __global__ void k_device_math(int fn, const double* x, int64_t n, double* y) {
 }
 
 // brick of an OK cell (index (bz nby + by) nbx + bx over the cell bounding box); -1 for other cells
-__device__ __forceinline__ int64_t cell_brick(uint64_t key, int lx, int ly, int lz, int nbx, int nby) {
+__device__ __forceinline__ int64_t cell_brick(uint64_t key, int lx, int ly, int lz, int nbx, int nby, int sh) {
   int cx, cy, cz;
   unpack_key(key, cx, cy, cz);
-  return ((int64_t)((cz - lz) >> kBrickShift) * nby + ((cy - ly) >> kBrickShift)) * nbx + ((cx - lx) >> kBrickShift);
+  return ((int64_t)((cz - lz) >> sh) * nby + ((cy - ly) >> sh)) * nbx + ((cx - lx) >> sh);
 }
 
 // per-brick counts of OK cells, and each cell's rank within its brick
 __global__ void k_brick_count(const uint64_t* cell_key, const int32_t* status, int64_t G, int lx, int ly, int lz,
-                              int nbx, int nby, int64_t* bcnt, int32_t* rank) {
+                              int nbx, int nby, int sh, int64_t* bcnt, int32_t* rank) {
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= G) return;
   if (status[g] != KSDF_CELL_OK) {
     rank[g] = -1;
     return;
   }
-  const int64_t b = cell_brick(cell_key[g], lx, ly, lz, nbx, nby);
+  const int64_t b = cell_brick(cell_key[g], lx, ly, lz, nbx, nby, sh);
   rank[g] = (int32_t)atomicAdd((unsigned long long*)&bcnt[b], 1ull);
 }
 
 __global__ void k_brick_fill(const uint64_t* cell_key, const int32_t* rank, int64_t G, int lx, int ly, int lz,
-                             int nbx, int nby, const int64_t* boff, int32_t* cells) {
+                             int nbx, int nby, int sh, const int64_t* boff, int32_t* cells, uint64_t* keys) {
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= G || rank[g] < 0) return;
-  cells[boff[cell_brick(cell_key[g], lx, ly, lz, nbx, nby)] + rank[g]] = (int32_t)g;
+  const uint64_t k = cell_key[g];
+  const int64_t i = boff[cell_brick(k, lx, ly, lz, nbx, nby, sh)] + rank[g];
+  cells[i] = (int32_t)g;
+  keys[i] = k;
 }
 
 ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const float* nrm, int64_t S, const Model* prev,
@@ -1835,26 +1838,34 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
   // bricks over the cell bounding box for the candidate search (OK cells only; statuses are final here)
   {
     int64_t nbk[3];
-    for (int j = 0; j < 3; ++j) {
-      nbk[j] = (((int64_t)hb[3 + j] - hb[j]) >> kBrickShift) + 1;
-      m.bk_lo[j] = hb[j];
+    int64_t nb = 0;
+    bool fits = false;
+    for (int sh = kBrickShift; sh <= kBrickShift + 1 && !fits; ++sh) {
+      nb = 1;
+      for (int j = 0; j < 3; ++j) {
+        nbk[j] = (((int64_t)hb[3 + j] - hb[j]) >> sh) + 1;
+        m.bk_lo[j] = hb[j];
+        nb *= nbk[j];
+      }
+      m.bk_shift = sh;
+      fits = nb <= 4 * G + 4096;
     }
-    const int64_t nb = nbk[0] * nbk[1] * nbk[2];
     m.nbricks = 0;
-    if (nb <= 4 * G + 4096) {
+    if (fits) {
       for (int j = 0; j < 3; ++j) m.bk_n[j] = (int)nbk[j];
       m.nbricks = nb;
       KSDF_CUDA(c, ensure(m.bk_off, sizeof(int64_t) * (nb + 1)));
       KSDF_CUDA(c, ensure(m.bk_cells, sizeof(int32_t) * G));
+      KSDF_CUDA(c, ensure(m.bk_keys, sizeof(uint64_t) * G));
       KSDF_CUDA(c, ensure(c->ws[WS_BRICK], sizeof(int32_t) * G));
       int64_t* boff = ptr<int64_t>(m.bk_off);
       int32_t* rank = ptr<int32_t>(c->ws[WS_BRICK]);
       KSDF_CUDA(c, cudaMemsetAsync(boff, 0, sizeof(int64_t) * (nb + 1), st));
       launch(k_brick_count, ceil_div(G, 256), 256, 0, st, ptr<uint64_t>(m.key), ptr<int32_t>(m.status), G, hb[0],
-             hb[1], hb[2], m.bk_n[0], m.bk_n[1], boff, rank);
+             hb[1], hb[2], m.bk_n[0], m.bk_n[1], m.bk_shift, boff, rank);
       KSDF_CUDA(c, scan_i64(boff, boff, nb, boff + nb, c->ws[WS_SCAN], st));
       launch(k_brick_fill, ceil_div(G, 256), 256, 0, st, ptr<uint64_t>(m.key), rank, G, hb[0], hb[1], hb[2],
-             m.bk_n[0], m.bk_n[1], boff, ptr<int32_t>(m.bk_cells));
+             m.bk_n[0], m.bk_n[1], m.bk_shift, boff, ptr<int32_t>(m.bk_cells), ptr<uint64_t>(m.bk_keys));
     }
   }
   KSDF_CUDA(c, cudaMemcpyAsync(hmax, dmax, sizeof(hmax), cudaMemcpyDeviceToHost, st));

@@ -19,7 +19,7 @@ constexpr int kMaxPre = 8192;           // collection-box members before the cap
 constexpr int kMaxK = 32;               // candidate list length limit
 constexpr int kMaxNmax = 512;           // training-set cap limit
 constexpr uint64_t kEmptyKey = ~0ull;   // empty hash slot
-constexpr int kBrickShift = 3;          // bricks of 8 cells per axis
+constexpr int kBrickShift = 2;          // bricks of 4 cells per axis, 8 where the box is too sparse for that
 constexpr unsigned kWaitLimit = 1u << 26;  // bounded spin on an mbarrier (~seconds)
 
 // device status word bits (ksdf_sync_status)
@@ -205,12 +205,13 @@ struct Model {
                    // contraction, rows (N dim) padded to Np = 16 ceil(N/16), columns (K dim) to Kp = 8 ceil(N/8),
                    // in K-quads: element (j, i) at (i / 4) Np 4 + j 4 + i % 4 (zero outside the lower triangle),
                    // FP32 (split into TF32 hi and lo parts in shared memory by the query)
-  // bricks of 2^kBrickShift cells per axis over the cell bounding box, each listing its OK cells (the
+  // bricks of 2^bk_shift cells per axis over the cell bounding box, each listing its OK cells (the
   // coarse level of the candidate search for query bins far from the nearest cells); nbricks = 0 when the
   // box is too sparse for a dense brick grid
   DevBuf bk_off;    // int64 (nbricks + 1), brick index (bz nby + by) nbx + bx
   DevBuf bk_cells;  // int32 cell ids grouped by brick
-  int bk_lo[3] = {0, 0, 0}, bk_n[3] = {0, 0, 0};
+  DevBuf bk_keys;   // uint64 their keys
+  int bk_lo[3] = {0, 0, 0}, bk_n[3] = {0, 0, 0}, bk_shift = kBrickShift;
   int64_t nbricks = 0;
   // refit scheduling (Sec. IV-C, App. G), per cell (int32): the query counter c0 (requests as a fused candidate,
   // capped, halved when the cell is fitted), the training marks c2 (updates that changed the cell's training set
