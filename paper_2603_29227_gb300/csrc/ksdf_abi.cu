@@ -100,7 +100,7 @@ static void prof_fold(ksdf_ctx* c) {
   c->pending.clear();
 }
 
-cudaError_t fork_streams(ksdf_ctx* c) {
+cudaError_t fork_streams(ksdf_ctx* c, int n) {
   cudaError_t e = cudaSuccess;
   if (!c->aux[0]) {
     for (int i = 0; i < ksdf_ctx::kNumAux && e == cudaSuccess; ++i) e = cudaStreamCreateWithFlags(&c->aux[i], cudaStreamNonBlocking);
@@ -116,16 +116,18 @@ cudaError_t fork_streams(ksdf_ctx* c) {
     if (e != cudaSuccess) return e;
   }
   e = cudaEventRecord(c->ev_fork, c->stream);
-  for (int i = 0; i < ksdf_ctx::kNumAux && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(c->aux[i], c->ev_fork, 0);
+  for (int i = 0; i < n && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(c->aux[i], c->ev_fork, 0);
+  if (n < ksdf_ctx::kNumAux) return e;
   for (int i = 0; i < ksdf_ctx::kNumAux && e == cudaSuccess; ++i) e = cudaStreamWaitEvent(c->aux_hi[i], c->ev_fork, 0);
   return e;
 }
 
-cudaError_t join_streams(ksdf_ctx* c) {
+cudaError_t join_streams(ksdf_ctx* c, int n) {
   cudaError_t e = cudaSuccess;
-  for (int i = 0; i < ksdf_ctx::kNumAux && e == cudaSuccess; ++i) {
+  for (int i = 0; i < n && e == cudaSuccess; ++i) {
     e = cudaEventRecord(c->ev_join[i], c->aux[i]);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, c->ev_join[i], 0);
+    if (n < ksdf_ctx::kNumAux) continue;
     if (e == cudaSuccess) e = cudaEventRecord(c->ev_join_hi[i], c->aux_hi[i]);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(c->stream, c->ev_join_hi[i], 0);
   }

@@ -725,7 +725,7 @@ ksdf_status run_backward(ksdf_ctx* c, const float* xq, int64_t Q, const int8_t* 
   const int maxn = std::max(m.max_n, 1), bound = std::min(maxn, small ? kBwSmemN : kBwSplitN);
   launch(k_bw_cells, ceil_div(G, 256), 256, 0, st, cnt, ptr<int32_t>(m.n), G, bound, list, ccnt);
   const bool two = maxn > bound;
-  if (two) KSDF_CUDA(c, fork_streams(c));
+  if (two) KSDF_CUDA(c, fork_streams(c, 1));
   for (int part = two ? 1 : 0; part >= 0; --part) {
     const bool sm = small && part == 0;
     const size_t smem2 = bw_smem_bytes(part == 0 ? bound : maxn, sm);
@@ -752,7 +752,7 @@ ksdf_status run_backward(ksdf_ctx* c, const float* xq, int64_t Q, const int8_t* 
     const int64_t grid2 = std::min<int64_t>(std::min<int64_t>(G, Q), (int64_t)std::max(1, occ2) * c->num_sms);
     launch(kc, (unsigned)grid2, threads, smem2, part == 0 ? st : c->aux[0], ca, p);
   }
-  if (two) KSDF_CUDA(c, join_streams(c));
+  if (two) KSDF_CUDA(c, join_streams(c, 1));
   KSDF_CUDA(c, cudaGetLastError());
   prof_end(c, e0, "backward.cell");
   prof_end(c, e_b, "backward");

@@ -302,8 +302,10 @@ const FitTable& fit_table(int i);
 ksdf_status autotune_fit(ksdf_ctx* c, int* chosen, double* ms);
 
 // ---- fork/join of the context stream with the auxiliary streams (ksdf_abi.cu) ----
-cudaError_t fork_streams(ksdf_ctx* c);
-cudaError_t join_streams(ksdf_ctx* c);
+// with n < kNumAux the first n streams only, without the high-priority ones: all of them take some fifty calls, which a
+// small batch's adjoint waits for
+cudaError_t fork_streams(ksdf_ctx* c, int n = ksdf_ctx::kNumAux);
+cudaError_t join_streams(ksdf_ctx* c, int n = ksdf_ctx::kNumAux);
 
 // ---- sorting and scanning (ksdf_sort.cu) ----
 // exclusive scan of n int64 values (in may equal out); total (optional) gets the sum on the device.  With
