@@ -459,6 +459,13 @@ ksdf_status ksdf_autotune(ksdf_ctx* c, int* table, double* fit_ms) {
 
 int ksdf_autotune_tables(void) { return fit_table_count(); }
 
+// for the tests only, not part of include/ksdf.h: later fits take size-class table `table`, as after ksdf_autotune chose it
+ksdf_status ksdf_test_fit_table(ksdf_ctx* c, int table) {
+  if (!c || table < 0 || table >= fit_table_count()) return KSDF_ERR_ARG;
+  c->fit_tab = table;
+  return KSDF_OK;
+}
+
 int ksdf_autotune_query_configs(void) { return query_tune_count(); }
 
 ksdf_status ksdf_autotune_query(ksdf_ctx* c, const float* xq, int64_t Q, const int8_t* sign, int* choice,
