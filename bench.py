@@ -152,6 +152,20 @@ def oracle_stats(w, sel, fit_s, qb_s, threads):
             "extrapolated_how": "one fit + the sample's per-query time x all queries of the workload"}
 
 
+def compact(v, top=True):
+    """v as it is printed: floats inside the blocks to six digits, arrays of more than 16 numbers as their mean, smallest,
+    largest and last.  (The line is read from the end of a run's output; with a value per frame of the 100-frame streams
+    it had grown past 20 KB and its start was lost.)"""
+    if isinstance(v, dict):
+        return {k: compact(u, top and not isinstance(u, (dict, list, tuple))) for k, u in v.items()}
+    if isinstance(v, (list, tuple)):
+        if len(v) > 16 and all(isinstance(u, (int, float)) for u in v):
+            v = {"mean_min_max_last": [float(np.mean(v)), min(v), max(v), v[-1]]}
+            return compact(v, False)
+        return [compact(u, False) for u in v]
+    return v if top or not isinstance(v, float) else float("%.6g" % v)
+
+
 def run_reference(args):
     rank, world, _ = dist_env()
     if rank != 0:
@@ -435,7 +449,7 @@ def other_configs(torch, dev, ksdf, main_name):
     for mode, budget in (("exact", 0), ("scheduled", CITY_REFIT_BUDGET)):
         m = ksdf.KernelSDF(city.params)
         ksdf.ksdf_set_schedule(m.h, budget, 1e-3)
-        rec = {"refit_ms": [], "query_ms": [], "cells_refit": [], "cells": [], "samples": []}
+        rec = {"refit_ms": [], "query_ms": [], "cells_refit": [], "cells": []}
         S = 0
         for f in range(n_frames):
             hx, hv, hn = (t(a) for a in scans[f])
@@ -457,19 +471,17 @@ def other_configs(torch, dev, ksdf, main_name):
             rec["query_ms"].append(round(e[1].elapsed_time(e[2]), 3))
             rec["cells_refit"].append(nref)
             rec["cells"].append(int(ksdf.ksdf_model_size(m.h)[0]))
-            rec["samples"].append(S)
         upd = slice(1, None)
         tot = sum(rec["refit_ms"][upd]) + sum(rec["query_ms"][upd])
-        rec["queries_per_s_incl_refit"] = 1e6 * (n_frames - 1) / (tot * 1e-3)
-        rec["refit_ms_mean"] = float(np.mean(rec["refit_ms"][upd]))
-        rec["query_ms_mean"] = float(np.mean(rec["query_ms"][upd]))
-        rec["refit_budget"] = budget
-        streams[mode] = rec
+        streams[mode] = {"queries_per_s_incl_refit": 1e6 * (n_frames - 1) / (tot * 1e-3),
+                         "refit_ms_mean": float(np.mean(rec["refit_ms"][upd])), "refit_ms_max": max(rec["refit_ms"][upd]),
+                         "query_ms_mean": float(np.mean(rec["query_ms"][upd])), "query_ms_max": max(rec["query_ms"][upd]),
+                         "cells_refit_mean": float(np.mean(rec["cells_refit"][upd])), "cells_final": rec["cells"][-1],
+                         "samples_final": S, "refit_budget": budget}
         del m
     res["city_stream"] = {"workload": "100x100 m city block, %d frames of a 64x2048 LiDAR scan (~125k hits each, range "
                                       "noise 0.02 m) on a closed path, 1M queries per frame in the 40x40x6 m box "
-                                      "around the pose; the GP is fed the raw hits (the BHM front-end runs on the same "
-                                      "frames in city_frontend)" % n_frames,
+                                      "around the pose; the GP is fed the raw hits" % n_frames,
                           "exact": streams["exact"], "scheduled": streams["scheduled"]}
     res["city_frontend"] = city_frontend(torch, dev, city, scans)
     return res
@@ -566,17 +578,17 @@ def city_frontend(torch, dev, city, scans):
     F = len(scans)
     tot_ms = sum(rec["update_ms"]) + sum(rec["march_ms"]) + sum(rec["sign_ms"])
     pipeline = city_pipeline(torch, dev, city, scans, 20)
-    out = {"workload": "the city stream's %d LiDAR frames through the BHM map (hinge spacing 0.175 m, 8^3 hinges "
-                       "per block, l = 0.11 m, free samples every 0.175 m, 2 EM rounds, marching at 0.0875 m); per "
-                       "frame: update, surface points, sign of the 1M queries" % F,
+    out = {"workload": "the city stream's %d frames through the BHM map (hinges 0.175 m, 2 EM rounds, marching at "
+                       "0.0875 m); per frame: update, surface points, sign of the 1M queries" % F,
            "frames_per_s": F / (tot_ms * 1e-3), "hits_per_s": hits_total / (tot_ms * 1e-3),
            "samples_per_s_update": sum(rec["samples"]) / (sum(rec["update_ms"]) * 1e-3),
-           "update_ms_mean": float(np.mean(rec["update_ms"])), "march_ms_mean": float(np.mean(rec["march_ms"])),
+           "update_ms_mean": float(np.mean(rec["update_ms"])), "update_ms_max": max(rec["update_ms"]),
+           "march_ms_mean": float(np.mean(rec["march_ms"])), "march_ms_max": max(rec["march_ms"]),
            "sign_ms_mean": float(np.mean(rec["sign_ms"])),
            "samples_per_frame": float(np.mean(rec["samples"])),
            "features_per_sample": float(np.sum(rec["features"]) / max(1, np.sum(rec["samples"]))),
            "points_per_frame": float(np.mean(rec["points"])), "blocks_final": rec["blocks"][-1],
-           "tau_final": m.tau, "pipeline": pipeline, "per_frame": rec}
+           "tau_final": m.tau, "pipeline": pipeline}
     # the oracle on a bounded sample: 1,200 hits of frame 0 within 10 m of the sensor
     try:
         from oracle import bhm as obhm
@@ -638,7 +650,7 @@ def parity_block(w, sel, ref, om, got):
             "grad_angle_max_deg": float(ang[gsel].max()) if gsel.any() else 0.0,
             "grad_medial_excluded": int(np.sum(fin & (ratio < 1e-2))),
             "var_sdf_max_rel": float(vs[fin].max()), "var_f_max_scaled": float(vf[fin].max()),
-            "note": "per-query checks at every size are the GPU tests (tests/test_gpu_full.py)"}
+            "note": "every size: tests/test_gpu_full.py"}
 
 
 def main():
@@ -791,8 +803,7 @@ def main():
     roof["kernel"] = "query + adjoint (all their kernels, one CUDA graph)"
     roof["traffic"] = recorded_traffic()
     roof["algorithmic_bytes"] = both["hbm"]
-    roof["peak_source"] = ("probes of libksdf_peaks.so on this GPU (MUFU ex2, FP32 FFMA lane ops, tcgen05 TF32, "
-                           "FP64 DFMA), measured live; HBM: " + peak_src + " (of measured)")
+    roof["peak_source"] = "probes of libksdf_peaks.so, measured live; HBM: " + peak_src + " (of measured)"
     rooflines = {"query": roofline_of(fwd, per.get("query", qb_ms) * 1e-3, P),
                  "adjoint": roofline_of(bwd, per.get("backward", qb_ms) * 1e-3, P)}
     if "fit.cholesky" in per and "fp64" in P:
@@ -800,9 +811,9 @@ def main():
         rooflines["fit.cholesky"] = {"bound": "alu", "unit": "TFLOP/s (FP64)",
                                      "achieved": fl64 / (per["fit.cholesky"] * 1e-3) / 1e12, "peak": P["fp64"] / 1e12,
                                      "nominal_peak": 1.25,
-                                     "what": "FP64 flops of the factorisation: N^3/3 + 2 N^2 per cell, over the "
-                                             "factorisation stage, which also runs most of the FP32 L^-1 kernels "
-                                             "(high-priority streams beside the FP64 classes)",
+                                     "what": "flops of the factorisation, N^3/3 + 2 N^2 per cell, against the FP64 "
+                                             "probe (cells within the fixed-point range run on the integer pipe, so 1 "
+                                             "is no bound); the stage also runs most of the FP32 L^-1 kernels",
                                      "stage_ms": per["fit.cholesky"], "linv_tail_ms": per.get("fit.linv")}
         rooflines["fit.cholesky"]["frac"] = rooflines["fit.cholesky"]["achieved"] / rooflines["fit.cholesky"]["peak"]
 
@@ -876,15 +887,13 @@ def main():
 
     cfg = workload_config(w, args)  # the same block as the reference arm's
     run = {"cells": int(len(nsz)), "work": wstats,
-                "launch": ("fit launched from the host (it sizes its launches on the host); query + adjoint replayed "
-                           "from one CUDA graph captured after the warm-up" if not args.no_graph
+                "launch": ("fit launched from the host; query + adjoint replayed from one CUDA graph" if not args.no_graph
                            else "all launched from the host"),
                 "fit_autotune": {"table": tune_idx, "fit_ms_per_table": [round(float(v), 3) for v in tune_ms]},
                 "query_autotune": {"choice": qtune_idx, "query_ms_per_pair": [round(float(v), 3) for v in qtune_ms],
-                                   "pairs": "3 x phase A budget (64, 128, 256 chunks) + phase B class split (64, "
-                                            "96, 128 samples)"},
-                "precision": "FP64 kernel matrix (entries above 2.4e-16; smaller ones in FP32), Cholesky and alpha; "
-                             "FP32 L^-1; FP32 query with compensated mean; V[f] contraction on tcgen05 in TF32 split "
+                                   "pairs": "3 x phase A budget (64, 128, 256) + phase B split (64, 96, 128)"},
+                "precision": "FP64 kernel matrix (entries above 2.4e-16; smaller ones in FP32); Cholesky in 64-bit fixed "
+                             "point (FP64 outside its range), alpha in FP64; FP32 L^-1; FP32 query with compensated mean; V[f] contraction on tcgen05 in TF32 split "
                              "three ways with FP32 accumulation; FP32 adjoint with one FP64 refinement of each cell "
                              "solve"}
     line = {
@@ -917,7 +926,7 @@ def main():
         torch.cuda.empty_cache()
         line["other_configs"] = other_configs(torch, dev, ksdf, w.name)
         line["other_configs"][w.name + "_var_grad"] = vg
-    print(json.dumps(line), flush=True)
+    print(json.dumps(compact(line)), flush=True)
     if world > 1:
         torch.distributed.destroy_process_group()
     return 0
