@@ -123,10 +123,14 @@ ksdf_status ksdf_set_stream(ksdf_ctx* ctx, void* stream);
 ksdf_status ksdf_reserve(ksdf_ctx* ctx, int64_t max_samples, int64_t max_queries);
 
 /* Fit (Sec. IV-B.1): bin the S samples x (S x dim, float64) into cells, assemble every cell's training
- * set from its collection box, build A = K + diag(sigma^2) (var: S float32 sigma_i^2 >= 0, NULL = 0) in
- * FP64, factor A = L L^T in FP64 and solve alpha = A^{-1} 1 in FP64 (kept in FP64 and FP32); L is kept in
+ * set from its collection box, build A = K + diag(sigma^2) (var: S float32 sigma_i^2 >= 0, NULL = 0) to FP64
+ * accuracy, factor A = L L^T and solve alpha = A^{-1} 1 (kept in FP64 and FP32); L is kept in
  * FP64 for the plain query and the adjoint, and L^{-1} is formed in FP32 from L for the mixed query's
- * variance contraction.  normals (S x dim
+ * variance contraction.  A cell whose variances all lie in [2^-20, 0.25] (sigma from 0.98 mm to 0.5 m) is factored
+ * in 64-bit fixed point: entries of A and sums to 2^-60, entries of L to 2^-57, alpha from L in FP64.  L and alpha
+ * are as close to exact arithmetic as the FP64 factorisation's, in norm; a single entry of L below 2^-5 has fewer
+ * than 53 significant bits.  One sample outside those bounds puts every cell that holds it on the FP64
+ * factorisation, which takes 1.5 (cells of 80 samples) to 4 times (470) as long.  normals (S x dim
  * float32, may be NULL) feed the sign stand-in.  Replaces any previous model.  Synchronises the stream
  * (cell counts decide allocation sizes).  Returns KSDF_ERR_NONFINITE for NaN/Inf/out-of-grid samples
  * or a negative variance, KSDF_ERR_CAPACITY if a collection box holds more than 8192 samples before
@@ -200,7 +204,8 @@ int ksdf_autotune_tables(void);
  * tensor-memory class (64, 96 or 128 samples; larger cells up to 256 take 256 columns).  Every pair
  * (ksdf_autotune_query_configs() of them, index = 3 x budget index + class index) runs the full query twice, the
  * second timed with CUDA events on the context's stream; the fastest is kept for the context's later queries.
- * The outputs do not depend on the choice.  *choice (may be NULL) gets the index, query_ms (may be NULL,
+ * (Every output of KSDF_OUT_ALL is asked for, the flags included; queries without them take less shared memory in
+ * phase A and might do best with another budget.)  The outputs do not depend on the choice.  *choice (may be NULL) gets the index, query_ms (may be NULL,
  * ksdf_autotune_query_configs() doubles) the times.  Synchronises the stream.  KSDF_ERR_NOT_FITTED without a
  * model, KSDF_ERR_ARG for Q <= 0. */
 ksdf_status ksdf_autotune_query(ksdf_ctx* ctx, const float* xq, int64_t Q, const int8_t* sign, int* choice,
@@ -231,7 +236,9 @@ ksdf_status ksdf_device_math(ksdf_ctx* ctx, int fn, const double* x, int64_t n, 
  * var_f[Q] (V[f], Sec. IV-B.1), var_grad[Q x dim] (only with KSDF_OUT_VAR_GRAD: V[grad_k u] of Sec. IV-B.3 /
  * App. C, the surface-sample variances propagated through the softmin's gradient on the winner; +inf for a
  * query on a sample, 0 without a GP), winner[Q] (cell id of the fused GP, -1 if none; keep it for the
- * backward), flags[Q] (KSDF_FLAG_*).  Outputs not selected may be NULL. */
+ * backward), flags[Q] (KSDF_FLAG_*).  Outputs not selected may be NULL.  The flags cost time: a near tie needs every
+ * candidate's u and its error bound, where a query without them leaves out the candidates that cannot win (phase A
+ * of 16,777,216 grid queries 6.05 against 3.74 ms); the other outputs are the same either way. */
 ksdf_status ksdf_query(ksdf_ctx* ctx, const float* xq, int64_t Q, const int8_t* sign, uint32_t out_mask, float* sdf,
                        float* grad, float* var_sdf, float* var_f, float* var_grad, int32_t* winner, uint32_t* flags);
 

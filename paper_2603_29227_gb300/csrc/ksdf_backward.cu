@@ -585,7 +585,7 @@ __global__ void __launch_bounds__(NT) k_bw_cell(BwCellArgs a, Params p) {
       const int k = k0 + tid;
       double c0 = 0.0, c1 = 0.0, c2 = 0.0, c3 = 0.0;  // four independent chains (DFMA latency ~64 cycles)
       // a warp walks rows from its first lane's column so that a row's loads coalesce; entries above the
-      // diagonal (k > i, read in bounds from the following row) are masked to zero
+      // diagonal (k > i) are not loaded and count as zero
       int i = k0 + (tid & ~31);
       if (k < n) {
         for (; i + 3 < n; i += 4) {

@@ -374,17 +374,17 @@ __global__ void k_sched_after(const int32_t* touched, int64_t G, int32_t* c0, in
   }
 }
 
-// The fit order's sort key of each cell (a warp per cell): cells for the fixed-point factorisation (fx allowed and
-// every sigma_i^2 within its bounds) by descending size, then the cells for the binary64 one by descending size,
+// The fit order's sort key of each cell (a warp per cell): cells for the fixed-point factorisation (every sigma_i^2
+// within its bounds) by descending size, then the cells for the binary64 one by descending size,
 // then the cells that are not fitted; hist[0 .. n_max] counts the first kind by size, hist[n_max + 1 ..] the second.
 __global__ void k_order_keys(const int32_t* n32, const int32_t* touched, const int64_t* ts_off, const float* mvar,
-                             int64_t G, int n_max, int fx, uint64_t* keys, uint32_t* vals, int* hist) {
+                             int64_t G, int n_max, uint64_t* keys, uint32_t* vals, int* hist) {
   const int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (g >= G) return;
   const int n = n32[g];
   const bool fit = !touched || touched[g];
-  bool ok = fx != 0 && n > 0;
+  bool ok = n > 0;
   if (fit && ok) {
     const float* v = mvar + ts_off[g];
     for (int i = lane; i < n; i += 32) ok &= v[i] >= kFxMinVar && v[i] <= kFxMaxVar;
@@ -793,7 +793,7 @@ __device__ void fit_lookahead(double* A, double* dinv, int N, int& s_fail, int& 
 //      team updates the trailing triangle in 2 x 2 register blocks over the panel depth.  The augmented row
 //      ends as y = L^{-1} 1.
 //   3. alpha = L^{-T} y by backward substitution (warp 0) while the other warps write L out.
-// L^{-1} in FP32 follows in k_linv.
+// L^{-1} in FP32 follows in k_linv_small or k_linv_big.
 template <int TEAM, bool GMAT>
 __global__ void __launch_bounds__(TEAM, TEAM == 32 ? 12 : 256 / TEAM) k_fit(FitArgs a, Params p) {
   constexpr int W = TEAM / 32;
@@ -1202,7 +1202,8 @@ __global__ void __launch_bounds__(32 * W) k_linv_small(LinvArgs a) {
 // for the finished rows (a thread four rows x two columns: eight 16- and 8-byte loads feed 32 FFMAs), one warp solves
 // the 32 x 32 triangle
 // (a lane per column), and the block is written in both layouts.  Every entry is the same sum in the same order
-// (ascending k) as in k_linv_small.
+// (ascending k) as in k_linv_small.  Of the tensor-core image a group's columns get the rows from their own 32 x 32 block
+// on; the rows above hold no entry of L^{-1} and are not written (the query does not load them).
 // Measured: 865 cells of mean N 473, 15.7 -> 3.8 ms (one CTA of 16 warps per cell on a global slot before); latency of
 // the row blocks' chain bounds it.  Classes up to 128 stay on k_linv_small (0.84 ms for 7,400 cells of N 96..127).
 constexpr int kLbThreads = 128;
@@ -1577,7 +1578,7 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
   launch(k_gather_members, ceil_div(G * p.n_max, 256), 256, 0, st, ptr<uint64_t>(m.key), ptr<int32_t>(m.n),
          ptr<int64_t>(m.ts_off), ptr<int32_t>(m.mpad), G, p, x, var, nrm, ptr<int32_t>(m.mgid), ptr<D4>(m.md4),
          ptr<float4>(m.mf4), ptr<float>(m.mvar), nrm ? ptr<float4>(m.mnrm) : nullptr);
-  // 5. the fit, largest cells first, three size classes on three streams
+  // 5. the fit: two kinds of cells in size classes, largest first, each class on one of the auxiliary streams
   KSDF_CUDA(c, ensure(c->ws[WS_A], sizeof(uint64_t) * (G + 1)));
   KSDF_CUDA(c, ensure(m.cell_order, sizeof(uint32_t) * (G + 1)));
   uint64_t* okeys = ptr<uint64_t>(c->ws[WS_A]);
@@ -1600,7 +1601,7 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
   int* dhist = ctr + 64;
   KSDF_CUDA(c, cudaMemsetAsync(ctr, 0, sizeof(int) * (64 + nh), st));
   launch(k_order_keys, ceil_div(G * 32, 256), 256, 0, st, ptr<int32_t>(m.n), touched, ptr<int64_t>(m.ts_off),
-         ptr<float>(m.mvar), G, p.n_max, 1, okeys, order, dhist);
+         ptr<float>(m.mvar), G, p.n_max, okeys, order, dhist);
   KSDF_CUDA(c, radix_sort_u64(okeys, order, G, bits_for((uint64_t)nh), c->ws[WS_SORT], st));
   // size classes from the counts by kind and size, launched concurrently, largest first; each class has its team size
   std::vector<int> hist((size_t)nh);
@@ -1706,7 +1707,6 @@ ksdf_status fit_model(ksdf_ctx* c, const double* x, const float* var, const floa
       x.gscr = nullptr;
       x.gstride = 0;
       x.np = np;
-      x.st = stw;
       const size_t smem = team == 32 ? 8 * (size_t)fx_elems(np + 1) : fx_team_smem(np, !cfg.gmat, team / 32);
       if (cfg.gmat) {
         x.gstride = fx_elems(np + 1);

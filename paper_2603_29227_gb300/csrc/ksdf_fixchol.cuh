@@ -1,8 +1,8 @@
 // ksdf_fixchol.cuh -- the Cholesky factorisation and the forward solve of the fit in 64-bit fixed point on the integer
 // pipe, and the backward solve (included by ksdf_fit.cu).
 //
-// Why: an SM of this part retires 1.9 FP64 FMA lanes per cycle but 28 lanes of 32 x 32 + 64 -> 64-bit integer
-// multiply-add (measured), and a GP's kernel matrix is the friendliest input fixed point can have: A = K + diag(s^2)
+// Why: an SM of this part retires 2.0 FP64 FMA lanes per cycle but 32 lanes of 32 x 32 + 64 -> 64-bit integer
+// multiply-add (measured: 0.63 and 10.0 T/s at 2070 MHz), and a GP's kernel matrix is the friendliest input fixed point can have: A = K + diag(s^2)
 // has a diagonal in [1, 1.25] and every entry of A, of its Schur complements and of L bounded by sqrt(1.25).  An FMA
 // on 57 fractional bits takes three integer multiply-adds, so the pipe's bound is five times the FP64 pipe's, and the
 // absolute rounding (2^-58 per entry of L, 2^-60 per sum) is below binary64's on these numbers: against 113-bit
@@ -50,7 +50,9 @@ __host__ __device__ inline size_t fx_team_smem(int np, bool smem_mat, int warps)
 }
 
 __device__ __forceinline__ long long fx_mad(int a, int b, long long c) {
-  long long r;  // written as a product and a sum: one multiply-add (mad.wide.s32 and C++ compile to a sum more)
+  // (a product and a sum in one asm statement: with mad.wide.s32 in it the factorisation of 81,700 cells of mean N 80 took
+  // 17.5 instead of 17.0 ms, with C++ arithmetic 18.6; of 865 cells of mean N 473 13.9 and 14.8 instead of 13.8)
+  long long r;
   asm("{.reg .s64 t; mul.wide.s32 t, %1, %2; add.s64 %0, t, %3;}" : "=l"(r) : "r"(a), "r"(b), "l"(c));
   return r;
 }
@@ -124,7 +126,6 @@ struct FixArgs {
   int2* gscr;      // per-CTA global slot (largest class)
   int64_t gstride;
   int np;
-  uint32_t* st;
 };
 
 // L as packed binary64 rows: thread t of nt takes the entries t, t + nt, ... (consecutive threads, consecutive entries)
