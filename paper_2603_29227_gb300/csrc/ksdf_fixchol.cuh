@@ -5,12 +5,13 @@
 // multiply-add (measured: 0.63 and 10.0 T/s at 2070 MHz), and a GP's kernel matrix is the friendliest input fixed point can have: A = K + diag(s^2)
 // has a diagonal in [1, 1.25] and every entry of A, of its Schur complements and of L bounded by sqrt(1.25).  An FMA
 // on 57 fractional bits takes three integer multiply-adds, so the pipe's bound is five times the FP64 pipe's, and the
-// absolute rounding (2^-58 per entry of L, 2^-60 per sum) is below binary64's on these numbers: against 113-bit
-// arithmetic alpha's relative error is 0.5 to 0.9 of the binary64 factorisation's (geometric means over cells of the
-// benchmark scenes), L's is the same (both carry the kernel entries' rounding).
+// absolute rounding (2^-58 per entry of L, 2^-60 per sum) is below binary64's on these numbers: against extended precision
+// alpha's largest relative error is 0.64 to 1.06 of the binary64 factorisation's (geometric means over 24 to 119 cells of
+// six maps, two groups above 1), L's root mean square error 0.40 to 0.99 (both carry the kernel entries' rounding).
 // Measured (with the L^-1 kernels that run beside it): 81,700 cells of mean N 80, 29.3 -> 19.0 ms; 865 cells of mean N
-// 473, 48.6 -> 12.4 ms; a stream frame with a tenth of its cells at N = 256, 34.4 -> 8.3 ms.  What bounds it now: the multiply-adds in the sums (about half of the pipe's rate, the
-// panels' serial 8 x 8 blocks take the rest), with shared memory allowing five to nine cells per SM.
+// 473, 48.6 -> 12.4 ms; a stream frame with a tenth of its cells at N = 256, 34.4 -> 8.3 ms.  What bounds it now: in the
+// largest class the multiply-adds (their pipe is 55% busy) and the two barriers around the panel's 8 x 8 block; in the teams
+// below the barriers; in the one-warp class the latency of the block's serial columns, at 7 to 8 warps per SM.
 //
 // Numbers.  "Q57 pair": v = h 2^27 + l with |l| <= 2^26 (two int32), value v 2^-57: L, y.  "Q60": int64, value 2^-60:
 // A, sums.  The product of two pairs is h h' 2^54 + (h l' + l h') 2^27 + l l' in units of 2^-114, i.e. h h' in Q60
