@@ -6,8 +6,9 @@
 // has a diagonal in [1, 1.25] and every entry of A, of its Schur complements and of L bounded by sqrt(1.25).  An FMA
 // on 57 fractional bits takes three integer multiply-adds, so the pipe's bound is five times the FP64 pipe's, and the
 // absolute rounding (2^-58 per entry of L, 2^-60 per sum) is below binary64's on these numbers: against extended precision
-// alpha's largest relative error is 0.64 to 1.06 of the binary64 factorisation's (geometric means over 24 to 119 cells of
-// six maps, two groups above 1), L's root mean square error 0.40 to 0.99 (both carry the kernel entries' rounding).
+// alpha's largest relative error is 0.76 to 1.02 of the binary64 factorisation's (geometric means over 24 to 119 cells of
+// each of six maps; one of them above 1), L's root mean square error 0.92 to 0.99 (both carry the kernel entries'
+// rounding).
 // Measured (with the L^-1 kernels that run beside it): 81,700 cells of mean N 80, 29.3 -> 19.0 ms; 865 cells of mean N
 // 473, 48.6 -> 12.4 ms; a stream frame with a tenth of its cells at N = 256, 34.4 -> 8.3 ms.  What bounds it now: in the
 // largest class the multiply-adds (their pipe is 55% busy) and the two barriers around the panel's 8 x 8 block; in the teams
